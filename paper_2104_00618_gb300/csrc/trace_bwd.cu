@@ -379,9 +379,14 @@ __global__ void __launch_bounds__(kTraceThreads, 2) trace_bwd_kernel(const __gri
   __shared__ uint2 s_lut[kSpreadLut];
   fill_spread_lut(s_lut);  // (its barrier also covers s_code_off)
 
+  // An item is one tile's pixels and item_cones of their cones (all or LPP),
+  // the cones being the outer index: the specular cones, the longest, first.
   for (;;) {
-    const int item = next_item(L.queue);
-    if (item >= L.total_tiles) break;
+    const int next = next_item(L.queue);
+    if (next >= L.total_items) break;
+    const int first = next / L.total_tiles * L.item_cones;
+    const int end = min(first + L.item_cones, n_cones);
+    const int item = next % L.total_tiles;
     int lo = 0, hi = L.n_views - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
@@ -458,7 +463,7 @@ __global__ void __launch_bounds__(kTraceThreads, 2) trace_bwd_kernel(const __gri
       tangent_frame(n, Tf, Bf);
       // The warp runs its lanes' cones together (the trip count is the same
       // for every lane: warp-collective operations inside need it).
-      for (int c0 = 0; c0 < n_cones; c0 += LPP) {
+      for (int c0 = first; c0 < end; c0 += LPP) {
         const int c = c0 + slot;
         const bool has_cone = c < n_cones;
         const ConeSel cs = select_cone(has_cone ? c : 0, L.spec_enable, L.occ_enable);

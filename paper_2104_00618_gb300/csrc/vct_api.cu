@@ -743,7 +743,19 @@ vct_status trace_backward_impl(const vct_pyramid *pyr, const vct_view *views,
   if (!workspace || workspace_bytes < need || !aligned(workspace, 256))
     return fail(VCT_ERR_WORKSPACE, "vct_trace_backward: workspace needs %llu bytes, 256-byte aligned",
                 (unsigned long long)need);
-  vct_launch_config c = cfg ? *cfg : vct_launch_config{8, 8, 1, 0};
+  const int sms = sm_count();
+  // Warps of a full chip (two CTAs of 256 threads per SM).
+  const int64_t resident = (int64_t)sms * 2 * (kTraceThreads / 32);
+  int64_t pixels = 0;
+  for (int i = 0; i < n_views; ++i) pixels += (int64_t)views[i].width * views[i].height;
+  // Tiles of 8 x 8 pixels; of 8 x 4, one round of a warp, where even those
+  // are fewer than half the warps of a full chip (all of them for the
+  // reproducible mode, whose rounds cost more).  Measured on a 64^3 grid
+  // with 8 cones, 8 x 8 / 8 x 4 tiles, each cone an item: 5917 pixels 302 /
+  // 223 us (reproducible 797 / 448), 32 400: 424 / 355 (718 / 449), 57 600:
+  // 420 / 451 (729 / 513), 129 600: 769 / 823 (875 / 849).
+  const bool few = pixels < 32 * (deterministic ? resident : resident / 2);
+  vct_launch_config c = cfg ? *cfg : vct_launch_config{8, few ? 4 : 8, 1, 0};
   if (!cfg_ok(c)) return fail(VCT_ERR_INVALID_ARG, "vct_trace_backward: bad launch config");
 
   auto L = std::make_unique<BwdLaunch>();
@@ -769,7 +781,6 @@ vct_status trace_backward_impl(const vct_pyramid *pyr, const vct_view *views,
   int per_sm = c.ctas_per_sm ? c.ctas_per_sm
                              : std::max(1, trace_bwd_occupancy(c.lanes_per_pixel, pyr->dtype,
                                                                L->pyr.bricked != 0));
-  const int sms = sm_count();
   for (int v0 = 0; v0 < n_views; v0 += kMaxBwdViewsPerLaunch) {
     const int nv = std::min(kMaxBwdViewsPerLaunch, n_views - v0);
     int cursor = 0;
@@ -783,9 +794,21 @@ vct_status trace_backward_impl(const vct_pyramid *pyr, const vct_view *views,
     }
     L->n_views = nv;
     L->total_tiles = cursor;
+    // With few tiles per warp, an item is lanes_per_pixel cones of a tile
+    // instead of all of them, so that a small launch fills the chip and a
+    // medium one ends evenly; with many, a tile's cones stay together.
+    // Measured as above, together / apart: 5917 pixels 637 / 302 us, 129 600:
+    // 866 / 769, 230 400: 1421 / 1225; 2.1 M pixels of a 128^3 grid, the
+    // whole training step: 13.4 / 14.6 ms (their cones' texels then reach
+    // the L1 at different times).
+    const int n_cones = params->n_diffuse + params->spec_enable + params->occ_enable;
+    const int groups = (n_cones + c.lanes_per_pixel - 1) / c.lanes_per_pixel;
+    const bool apart = cursor < 4 * resident;
+    L->item_cones = apart ? c.lanes_per_pixel : std::max(n_cones, 1);
+    L->total_items = apart ? cursor * groups : cursor;
     if (v0 > 0 && (e = cudaMemsetAsync(L->queue, 0, 4, s)) != cudaSuccess)
       return cuda_fail(e, "vct_trace_backward queue clear");
-    const int grid = std::max(1, std::min(cursor, per_sm * sms));
+    const int grid = std::max(1, std::min(L->total_items, per_sm * sms));
     e = launch_trace_bwd(*L, c.lanes_per_pixel, grid, s);
     if (e != cudaSuccess) return cuda_fail(e, "vct_trace_backward launch");
   }

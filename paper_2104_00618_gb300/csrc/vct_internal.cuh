@@ -337,6 +337,7 @@ struct BwdView {
 
 struct BwdLaunch {
   int n_views, total_tiles, tile_w, tile_h;
+  int total_items, item_cones;  // items: total_tiles x groups of item_cones cones
   int n_diffuse, spec_enable, occ_enable;
   int deterministic;  // 1: accumulate in 64-bit fixed point (gfix_lvl), not float
   int aniso;          // 1: anisotropic pyramid (gradient levels >= 1 hold six volumes)
