@@ -82,26 +82,40 @@ __device__ __forceinline__ void scatter_lane(const BwdLaunch &L, int l, uint32_t
 
 // Scatter of one level for the whole warp (warp-uniform call).  Lanes are
 // grouped by (level, 2x2x2 cell).  A lane whose group has fewer than
-// kReduceMin lanes scatters its own corners.  For each larger group the 32 values
-// (8 corners x 4 channels) are summed over the group by recursive halving,
-// so that lane j ends with the group total of value j, and each lane issues
-// one atomic on a distinct address: contending atomics (the same texel from
-// many lanes) are what makes a naive scatter slow at the coarse levels.
-// Measured on the learnable 128^3 workload (fwd + adjoint): 59.3 / 57.8 /
-// 55.4 / 53.7 / 57.1 / 91.2 ms for thresholds 2 / 4 / 8 / 16 / 20 / 32, and
-// 544 ms without the reduction.
-constexpr int kReduceMin = 16;
-// The reproducible mode pays four 64-bit atomics per corner and channel
-// group, so there every cell shared by two or more lanes is summed first
-// (fwd + adjoint on the same workload: 108.6 ms with 16, 64.7 ms with 2).
+// kReduceMin lanes scatters its own corners.  For each larger group the 32
+// sums (8 corners x 4 channels) over its lanes are dot products in shared
+// memory: lane i writes its corner weights (zeros outside the group) and its
+// derivatives as column i of the warp's rows, lane j reads weight row j / 4
+// against derivative row j % 4, four columns per pair of 16-byte loads, and
+// issues one atomic on a distinct address: contending atomics (the same
+// texel from many lanes) are what makes a naive scatter slow at the coarse
+// levels.  What binds is instruction issue and fixed latencies (ncu: 0.62 of
+// the issue peak, the atomics 3-10 % of the time): this form takes about 80
+// instructions per group, where the recursive halving by shuffles that it
+// replaces took 190.  Kernel on 8 views of 512^2, 128^3 grid: 7.70 G -> 6.5 G
+// warp instructions, the whole training step 13.45 -> 12.70 ms; the adjoint
+// alone, 2 views: 3.35 -> 2.77 ms (reproducible 4.52 -> 3.41, binary16 3.87
+// -> 2.92, anisotropic 64^3 4.00 -> 2.95).  Thresholds of 8 / 12 / 16 / 20
+// lanes: 13.0 / 12.75 / 13.0 / 14.3 ms per step.
+constexpr int kReduceMin = 12;
+// The reproducible mode pays four 64-bit atomics per corner, so there every
+// cell shared by two or more lanes is summed first.
 constexpr int kReduceMinFix = 2;
+
+// A warp's rows: 8 of corner weights, 4 of derivatives.  The row stride of 36
+// words places the 16-byte words of the weight rows at one column in
+// different banks.
+constexpr int kRowStride = 36;
+struct __align__(16) WarpRows {
+  float v[12][kRowStride];
+};
 
 // Slot of the key-offset table holding the total (after the per-level offsets).
 constexpr int kKeyTotal = VCT_MAX_LEVELS;
 
 template <bool AN>
 __device__ __forceinline__ void scatter_warp(const BwdLaunch &L, const uint32_t *code_off,
-                                             bool act, int l, uint32_t vbase, uint32_t lim,
+                                             WarpRows &rows, bool act, int l, uint32_t vbase, uint32_t lim,
                                              const LevelStencil &s, float lw, const float g[4]) {
   const unsigned full = 0xffffffffu;
   act = act && s.valid != 0u;  // a cell wholly outside the level has nothing to scatter
@@ -139,42 +153,43 @@ __device__ __forceinline__ void scatter_warp(const BwdLaunch &L, const uint32_t 
   if (act && !big) scatter_lane(L, l, vbase, lim, s, lw, g);
   unsigned pending = __ballot_sync(full, big);
   if (pending == 0u) return;
-  // A lane without a sample here holds unset fractions and derivatives: its
-  // operands are replaced by zeros once, so that every product below is of
-  // finite values and a lane outside a group adds exact zeros (level weight
-  // 0).  The weight is selected inside the loop, which also keeps the 32
-  // products from being hoisted out of it and held in registers.
-  const float fr[3] = {act ? s.fr[0] : 0.0f, act ? s.fr[1] : 0.0f, act ? s.fr[2] : 0.0f};
-  const float ga[4] = {act ? g[0] : 0.0f, act ? g[1] : 0.0f, act ? g[2] : 0.0f,
-                       act ? g[3] : 0.0f};
-  const float lwa = act ? lw : 0.0f;
+  // The columns of a group hold its lanes' weights, those of the other lanes
+  // zeros.  A lane without a sample here holds unset fractions and
+  // derivatives: zeros take their place.
+  float w[8];
+  {
+    const float fr[3] = {act ? s.fr[0] : 0.0f, act ? s.fr[1] : 0.0f, act ? s.fr[2] : 0.0f};
+    corner_weights(fr, act ? lw : 0.0f, w);
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) rows.v[8 + ch][lane] = act ? g[ch] : 0.0f;
+  }
+  const int c = lane >> 2, ch = lane & 3;
+  const float *wr = rows.v[c], *gr = rows.v[8 + ch];
+#pragma unroll 1
   while (pending) {
     const int leader = __ffs(pending) - 1;
     const unsigned lgrp = __shfl_sync(full, grp, leader);
     const bool in = (lgrp >> lane) & 1u;
-    float v[32];
-    {
-      float w[8];
-      corner_weights(fr, in ? lwa : 0.0f, w);
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
+    for (int k = 0; k < 8; ++k) rows.v[k][lane] = in ? w[k] : 0.0f;
+    __syncwarp();
+    f32x2 sum[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) v[4 * c + ch] = w[c] * ga[ch];
+    for (int k = 0; k < 32; k += 8) {
+      const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(wr + k);
+      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2 *>(gr + k);
+      const ulonglong2 a1 = *reinterpret_cast<const ulonglong2 *>(wr + k + 4);
+      const ulonglong2 b1 = *reinterpret_cast<const ulonglong2 *>(gr + k + 4);
+      sum[0] = f2_fma(a0.x, b0.x, sum[0]);
+      sum[1] = f2_fma(a0.y, b0.y, sum[1]);
+      sum[2] = f2_fma(a1.x, b1.x, sum[2]);
+      sum[3] = f2_fma(a1.y, b1.y, sum[3]);
     }
-#pragma unroll
-    for (int half = 16; half >= 1; half >>= 1) {
-      const bool upper = (lane & half) != 0;
-#pragma unroll
-      for (int i = 0; i < half; ++i) {
-        const float send = upper ? v[i] : v[i + half];
-        const float keep = upper ? v[i + half] : v[i];
-        v[i] = keep + __shfl_xor_sync(full, send, half);
-      }
-    }
-    // Lane j holds the group total of corner j / 4, channel j % 4.  The cell
-    // is the leader's: take its spread coordinates (a shuffle returns the
-    // source lane's value, so per-corner choices are made afterwards).
-    const int c = lane >> 2, ch = lane & 3;
+    const float2 p0 = f2_unpack(sum[0]), p1 = f2_unpack(sum[1]);
+    const float2 p2 = f2_unpack(sum[2]), p3 = f2_unpack(sum[3]);
+    const float v = ((p0.x + p0.y) + (p1.x + p1.y)) + ((p2.x + p2.y) + (p3.x + p3.y));
+    // The cell is the leader's: take its spread coordinates (a shuffle returns
+    // the source lane's value, so per-corner choices are made afterwards).
     const int ll = __shfl_sync(full, l, leader);  // this lane's own level may differ
     uint32_t lvbase = 0u, llim;
     if constexpr (AN) {
@@ -188,14 +203,15 @@ __device__ __forceinline__ void scatter_warp(const BwdLaunch &L, const uint32_t 
     const uint32_t sy0 = __shfl_sync(full, s.sy[0], leader), sy1 = __shfl_sync(full, s.sy[1], leader);
     const uint32_t sz0 = __shfl_sync(full, s.sz[0], leader), sz1 = __shfl_sync(full, s.sz[1], leader);
     const uint32_t idx =
-        lvbase + (((c & 1) ? sx1 : sx0) | (((c >> 1) & 1) ? sy1 : sy0) | ((c >> 2) ? sz1 : sz0));
-    if (((lvalid >> c) & 1u) && v[0] != 0.0f && in_bounds(idx, llim, kOobGrad)) {
+        lvbase + (((c & 1) ? sx1 : sx0) | ((c & 2) ? sy1 : sy0) | ((c & 4) ? sz1 : sz0));
+    if (((lvalid >> c) & 1u) && v != 0.0f && in_bounds(idx, llim, kOobGrad)) {
       if (L.deterministic)
-        atomicAdd(fix_texel(L, ll, idx) + ch, to_fix(v[0]));
+        atomicAdd(fix_texel(L, ll, idx) + ch, to_fix(v));
       else
-        atomicAdd(grad_texel(L, ll, idx) + ch, v[0]);
+        atomicAdd(grad_texel(L, ll, idx) + ch, v);
     }
     pending &= ~lgrp;
+    __syncwarp();  // the rows are written again
   }
 }
 
@@ -205,18 +221,18 @@ __device__ __forceinline__ void scatter_warp(const BwdLaunch &L, const uint32_t 
 // forward skipped none (warp-uniform trip count).
 template <bool AN>
 __device__ __forceinline__ void scatter_level(const BwdLaunch &L, const uint32_t *code_off,
-                                              bool act, int l, const LevelStencil &s, float lw,
+                                              WarpRows &rows, bool act, int l, const LevelStencil &s, float lw,
                                               const float g[4], const AnisoW &aw) {
   const uint32_t tex = (uint32_t)level_texels(L.pyr.n, l);
   if constexpr (!AN) {
-    scatter_warp<false>(L, code_off, act, l, 0u, tex, s, lw, g);
+    scatter_warp<false>(L, code_off, rows, act, l, 0u, tex, s, lw, g);
   } else {
     const bool dir = l >= 1;
 #pragma unroll 1
     for (int a = 0; a < 3; ++a) {
       const bool on = act && (dir ? aw.wt[a] >= kAnisoSkip : a == 0);
       if (__any_sync(0xffffffffu, on))
-        scatter_warp<true>(L, code_off, on, l, dir ? (uint32_t)aw.vol[a] * tex : 0u,
+        scatter_warp<true>(L, code_off, rows, on, l, dir ? (uint32_t)aw.vol[a] * tex : 0u,
                      dir ? 6u * tex : tex, s, dir ? lw * aw.wt[a] : lw, g);
     }
   }
@@ -235,7 +251,7 @@ __device__ __forceinline__ void scatter_level(const BwdLaunch &L, const uint32_t
 // (1 - a_k) R'_{k+1}.
 template <int DT, bool BR, bool kVar, bool AN = false>
 __device__ __forceinline__ void cone_adjoint(const BwdLaunch &L, const uint32_t *code_off,
-                                             const uint2 *lut, bool active,
+                                             WarpRows &rows, const uint2 *lut, bool active,
                                              const Apex &A, const float w[3],
                                              const ConeConst &cc, float T0, float gc0, float gc1,
                                              float gc2, float ga, const uint2 *state, int mode) {
@@ -349,9 +365,9 @@ __device__ __forceinline__ void cone_adjoint(const BwdLaunch &L, const uint32_t 
       Q *= om;
       tr_next = tr;
     }
-    scatter_level<AN>(L, code_off, act, lp.l0, st[0], 1.0f - lp.f, g, aw);
+    scatter_level<AN>(L, code_off, rows, act, lp.l0, st[0], 1.0f - lp.f, g, aw);
     const bool two = act && lp.f > 0.0f;
-    if (__any_sync(full, two)) scatter_level<AN>(L, code_off, two, lp.l1, st[1], lp.f, g, aw);
+    if (__any_sync(full, two)) scatter_level<AN>(L, code_off, rows, two, lp.l1, st[1], lp.f, g, aw);
   }
 }
 
@@ -377,6 +393,7 @@ __global__ void __launch_bounds__(kTraceThreads, 2) trace_bwd_kernel(const __gri
     s_code_off[kKeyTotal] = acc;
   }
   __shared__ uint2 s_lut[kSpreadLut];
+  __shared__ WarpRows s_rows[kTraceThreads / 32];
   fill_spread_lut(s_lut);  // (its barrier also covers s_code_off)
 
   // An item is one tile's pixels and item_cones of their cones (all or LPP),
@@ -409,61 +426,63 @@ __global__ void __launch_bounds__(kTraceThreads, 2) trace_bwd_kernel(const __gri
       const bool inimg = pi < tile_pix && px < V.W && py < V.H;
       const int p = inimg ? py * V.W + px : 0;
       const bool pix_on = inimg && (V.mask == nullptr || V.mask[p] != 0);
-      float x[3] = {0.f, 0.f, 0.f}, n[3] = {0.f, 0.f, 1.f};
-      float4 gD = make_float4(0.f, 0.f, 0.f, 0.f), gS = gD;
-      float gV = 0.f;
-      if (pix_on) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          x[a] = V.pos[3 * p + a];
-          n[a] = V.nrm[3 * p + a];
-        }
-        if (BV.gD) gD = reinterpret_cast<const float4 *>(BV.gD)[p];
-        if (BV.gS) gS = reinterpret_cast<const float4 *>(BV.gS)[p];
-        if (BV.gV) gV = BV.gV[p];
-        if (BV.gL && (L.var.flags & VCT_FLAG_SHADE)) {
-          // chain rule through the shading epilogue: L_ch depends on D_ch,
-          // S_ch and Vis (L_vxct = alb (kd D + ks S) + Vis direct; L_impl =
-          // Vis (D + direct) + S, which needs the forward's D and Vis)
-          const float4 gL = reinterpret_cast<const float4 *>(BV.gL)[p];
-          float direct[3], alb[3];
-          shade_direct(L.var, V, p, direct, alb);
-          const float gl[3] = {gL.x, gL.y, gL.z};
-          float dD[3], dS[3], dV = 0.f;
-          if (L.var.flags & VCT_FLAG_SHADE_IMPL) {
-            const float4 Df = reinterpret_cast<const float4 *>(V.outD)[p];
-            const float vis = (L.occ_enable && V.outV) ? V.outV[p] : 1.0f;
-            const float Dc[3] = {Df.x, Df.y, Df.z};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              dD[a] = gl[a] * vis;
-              dS[a] = gl[a];
-              dV = fmaf(gl[a], Dc[a] + direct[a], dV);
-            }
-          } else {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              dD[a] = gl[a] * alb[a] * L.var.kd;
-              dS[a] = gl[a] * alb[a] * L.var.ks;
-              dV = fmaf(gl[a], direct[a], dV);
-            }
-          }
-          gD.x += dD[0];
-          gD.y += dD[1];
-          gD.z += dD[2];
-          gS.x += dS[0];
-          gS.y += dS[1];
-          gS.z += dS[2];
-          gV += dV;
-        }
-      }
-      Apex A;
-      make_apex(P, x, n, L.normal_offset, A);
-      float Tf[3], Bf[3];
-      tangent_frame(n, Tf, Bf);
       // The warp runs its lanes' cones together (the trip count is the same
       // for every lane: warp-collective operations inside need it).
       for (int c0 = first; c0 < end; c0 += LPP) {
+        // (the pixel is set up anew for each cone: its position, frame and
+        // upstream gradients would hold some 20 registers across the walk)
+        float x[3] = {0.f, 0.f, 0.f}, n[3] = {0.f, 0.f, 1.f};
+        float4 gD = make_float4(0.f, 0.f, 0.f, 0.f), gS = gD;
+        float gV = 0.f;
+        if (pix_on) {
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            x[a] = V.pos[3 * p + a];
+            n[a] = V.nrm[3 * p + a];
+          }
+          if (BV.gD) gD = reinterpret_cast<const float4 *>(BV.gD)[p];
+          if (BV.gS) gS = reinterpret_cast<const float4 *>(BV.gS)[p];
+          if (BV.gV) gV = BV.gV[p];
+          if (BV.gL && (L.var.flags & VCT_FLAG_SHADE)) {
+            // chain rule through the shading epilogue: L_ch depends on D_ch,
+            // S_ch and Vis (L_vxct = alb (kd D + ks S) + Vis direct; L_impl =
+            // Vis (D + direct) + S, which needs the forward's D and Vis)
+            const float4 gL = reinterpret_cast<const float4 *>(BV.gL)[p];
+            float direct[3], alb[3];
+            shade_direct(L.var, V, p, direct, alb);
+            const float gl[3] = {gL.x, gL.y, gL.z};
+            float dD[3], dS[3], dV = 0.f;
+            if (L.var.flags & VCT_FLAG_SHADE_IMPL) {
+              const float4 Df = reinterpret_cast<const float4 *>(V.outD)[p];
+              const float vis = (L.occ_enable && V.outV) ? V.outV[p] : 1.0f;
+              const float Dc[3] = {Df.x, Df.y, Df.z};
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                dD[a] = gl[a] * vis;
+                dS[a] = gl[a];
+                dV = fmaf(gl[a], Dc[a] + direct[a], dV);
+              }
+            } else {
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                dD[a] = gl[a] * alb[a] * L.var.kd;
+                dS[a] = gl[a] * alb[a] * L.var.ks;
+                dV = fmaf(gl[a], direct[a], dV);
+              }
+            }
+            gD.x += dD[0];
+            gD.y += dD[1];
+            gD.z += dD[2];
+            gS.x += dS[0];
+            gS.y += dS[1];
+            gS.z += dS[2];
+            gV += dV;
+          }
+        }
+        Apex A;
+        make_apex(P, x, n, L.normal_offset, A);
+        float Tf[3], Bf[3];
+        tangent_frame(n, Tf, Bf);
         const int c = c0 + slot;
         const bool has_cone = c < n_cones;
         const ConeSel cs = select_cone(has_cone ? c : 0, L.spec_enable, L.occ_enable);
@@ -504,7 +523,7 @@ __global__ void __launch_bounds__(kTraceThreads, 2) trace_bwd_kernel(const __gri
         const uint2 *st = V.state == nullptr ? nullptr
                           : V.state + (on ? (size_t)c * V.W * V.H + p : 0);
         if (__any_sync(0xffffffffu, on))
-          cone_adjoint<DT, BR, kVar, AN>(L, s_code_off, s_lut, on, A, w, cc, T0, g0, g1, g2, ga,
+          cone_adjoint<DT, BR, kVar, AN>(L, s_code_off, s_rows[threadIdx.x >> 5], s_lut, on, A, w, cc, T0, g0, g1, g2, ga,
                                          st, mode);
       }
     }
