@@ -189,6 +189,19 @@ vct_status vct_build_mips(const float *level0_dense, const vct_pyramid *pyr,
                           vct_stream_t stream);
 
 /*
+ * vct_build_mips of a VCT_LAYOUT_BRICKS pyramid right after
+ * vct_pyramid_plan_bricks: `scratch` still holds what that call left there
+ * for the same n, levels, dtype and level0_dense, whose contents are
+ * unchanged, and the occupancy is taken from it instead of from another pass
+ * over the grid.  Same result and errors as vct_build_mips, and
+ * VCT_ERR_INVALID_ARG for another layout, VCT_ERR_WORKSPACE for a NULL, too
+ * small or misaligned scratch (vct_pyramid_plan_scratch_bytes()).
+ */
+vct_status vct_build_mips_planned(const float *level0_dense, const vct_pyramid *pyr,
+                                  const void *scratch, size_t scratch_bytes,
+                                  vct_stream_t stream);
+
+/*
  * Copies level `level` of `pyr` into a dense float32 array
  * [m][m][m][4] (m = n >> level, z, y, x, channel) at `dense_out` (device).
  */

@@ -117,9 +117,8 @@ def _check_level0(level0):
                        "level0 must be a contiguous CUDA float32 tensor [n, n, n, 4]")
 
 
-def plan_bricks(level0: torch.Tensor, levels: int | None = None, dtype="f32",
-                stream=None) -> tuple[int, int]:
-    """(occupied bricks, bytes) of a brick pyramid of this grid (synchronises)."""
+def _plan_bricks(level0, levels, dtype, stream):
+    """(occupied bricks, bytes, the scratch that holds the plan)."""
     _check_level0(level0)
     n = level0.shape[0]
     levels = num_levels(n) if levels is None else int(levels)
@@ -130,7 +129,13 @@ def plan_bricks(level0: torch.Tensor, levels: int | None = None, dtype="f32",
     check(lib().vct_pyramid_plan_bricks(_ptr(level0), n, levels, dt, _ptr(scratch), sb,
                                         ctypes.byref(occ), ctypes.byref(nbytes),
                                         _stream(stream)), "vct_pyramid_plan_bricks")
-    return int(occ.value), int(nbytes.value)
+    return int(occ.value), int(nbytes.value), scratch
+
+
+def plan_bricks(level0: torch.Tensor, levels: int | None = None, dtype="f32",
+                stream=None) -> tuple[int, int]:
+    """(occupied bricks, bytes) of a brick pyramid of this grid (synchronises)."""
+    return _plan_bricks(level0, levels, dtype, stream)[:2]
 
 
 def build_mips(level0: torch.Tensor, levels: int | None = None, dtype="f32",
@@ -141,8 +146,15 @@ def build_mips(level0: torch.Tensor, levels: int | None = None, dtype="f32",
     _check_level0(level0)
     n = level0.shape[0]
     if out is None and LAYOUTS[layout] == _abi.LAYOUT_BRICKS:
-        occ, _ = plan_bricks(level0, levels, dtype, stream)
-        out = Pyramid(n, levels, dtype, origin, size, level0.device, "bricks", occ)
+        occ, _, scratch = _plan_bricks(level0, levels, dtype, stream)
+        pyr = Pyramid(n, levels, dtype, origin, size, level0.device, "bricks", occ)
+        p = pyr.struct()
+        check(lib().vct_build_mips_planned(_ptr(level0), ctypes.byref(p), _ptr(scratch),
+                                           scratch.numel(), _stream(stream)),
+              "vct_build_mips_planned")
+        if stream is not None:
+            scratch.record_stream(stream)  # allocated on the current stream
+        return pyr
     pyr = out if out is not None else Pyramid(n, levels, dtype, origin, size, level0.device,
                                               layout)
     p = pyr.struct()

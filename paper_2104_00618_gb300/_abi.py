@@ -117,6 +117,8 @@ EXPORTS = {
     "vct_pyramid_plan_bricks": (_c_i32, [_vp, _c_i32, _c_i32, _c_i32, _vp, ctypes.c_size_t,
                                          ctypes.POINTER(_c_u64), ctypes.POINTER(_c_u64), _vp]),
     "vct_build_mips": (_c_i32, [_vp, ctypes.POINTER(VctPyramid), _vp]),
+    "vct_build_mips_planned": (_c_i32, [_vp, ctypes.POINTER(VctPyramid), _vp, ctypes.c_size_t,
+                                        _vp]),
     "vct_pyramid_read_level": (_c_i32, [ctypes.POINTER(VctPyramid), _c_i32, _vp, _vp]),
     "vct_pyramid_status": (_c_i32, [ctypes.POINTER(VctPyramid), _vp]),
     "vct_trace_workspace_bytes": (ctypes.c_size_t, []),

@@ -428,7 +428,9 @@ uint64_t vct_pyramid_level_offset(int32_t n, int32_t levels, int32_t dtype, int3
   return make_layout(n, levels, dtype).level_off[level];
 }
 
-vct_status vct_build_mips(const float *level0_dense, const vct_pyramid *pyr, vct_stream_t stream) {
+// `planned`: tables of vct_pyramid_plan_bricks for this grid (brick layout), or null.
+static vct_status build_impl(const float *level0_dense, const vct_pyramid *pyr,
+                             const uint8_t *planned, vct_stream_t stream) {
   vct_status st = check_pyramid(pyr, "vct_build_mips");
   if (st != VCT_OK) return st;
   if (!level0_dense || !aligned(level0_dense, 16))
@@ -456,9 +458,27 @@ vct_status vct_build_mips(const float *level0_dense, const vct_pyramid *pyr, vct
                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(VCT_ERR_CUDA, "vct_build_mips: tensor map encode failed (%d)", (int)r);
-  cudaError_t e = launch_pack_mips(level0_dense, *pyr, &map, (cudaStream_t)stream);
+  cudaError_t e = launch_pack_mips(level0_dense, *pyr, &map, (cudaStream_t)stream, planned);
   if (e != cudaSuccess) return cuda_fail(e, "vct_build_mips launch");
   return VCT_OK;
+}
+
+vct_status vct_build_mips(const float *level0_dense, const vct_pyramid *pyr, vct_stream_t stream) {
+  return build_impl(level0_dense, pyr, nullptr, stream);
+}
+
+vct_status vct_build_mips_planned(const float *level0_dense, const vct_pyramid *pyr,
+                                  const void *scratch, size_t scratch_bytes,
+                                  vct_stream_t stream) {
+  vct_status st = check_pyramid(pyr, "vct_build_mips_planned");
+  if (st != VCT_OK) return st;
+  if (pyr->layout != VCT_LAYOUT_BRICKS)
+    return fail(VCT_ERR_INVALID_ARG, "vct_build_mips_planned: not a brick pyramid");
+  const Layout L = make_layout(pyr->n, pyr->levels, pyr->dtype, VCT_LAYOUT_BRICKS);
+  if (!scratch || scratch_bytes < L.pool_off || !aligned(scratch, 256))
+    return fail(VCT_ERR_WORKSPACE, "vct_build_mips_planned: scratch needs %llu bytes",
+                (unsigned long long)L.pool_off);
+  return build_impl(level0_dense, pyr, static_cast<const uint8_t *>(scratch), stream);
 }
 
 vct_status vct_pyramid_read_level(const vct_pyramid *pyr, int32_t level, float *dense_out,

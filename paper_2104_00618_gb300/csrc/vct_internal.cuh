@@ -393,8 +393,10 @@ vct_status set_last_error(vct_status st, const char *fmt, ...);
 bool streamed_build(const float *level0, const vct_pyramid &pyr);
 // `map`: the level-0 tensor map of the TMA path; unused (may be null) when
 // streamed_build() holds.
+// `planned`: see launch_brick_tables (brick pyramids).
 cudaError_t launch_pack_mips(const float *level0, const vct_pyramid &pyr,
-                             const CUtensorMap *map, cudaStream_t s);
+                             const CUtensorMap *map, cudaStream_t s,
+                             const uint8_t *planned = nullptr);
 cudaError_t launch_read_level(const vct_pyramid &pyr, int level, float *out, cudaStream_t s,
                               int direction = 0);
 cudaError_t launch_build_aniso(const float *level0, const vct_pyramid &pyr, int sms,
@@ -403,8 +405,11 @@ cudaError_t launch_build_aniso(const float *level0, const vct_pyramid &pyr, int 
 // level, written at layout L's table offsets from `base`; the occupied count
 // goes to base + kHeaderCountOff.  More than `capacity` bricks (zero brick
 // included) leaves every slot 0 and writes VCT_ERR_WORKSPACE to the status word.
+// `planned` (may be null): the base of tables made by an earlier call for the
+// same grid; they are copied instead of computed.
 cudaError_t launch_brick_tables(const float *level0, int n, int levels, const Layout &L,
-                                uint8_t *base, uint64_t capacity, cudaStream_t s);
+                                uint8_t *base, uint64_t capacity, cudaStream_t s,
+                                const uint8_t *planned = nullptr);
 cudaError_t launch_mip_adjoint(const float *gpyr_base, const Layout &gl, int n, int levels,
                                float *grad0, cudaStream_t s);
 // Adjoint of launch_build_aniso at the anisotropic pyramid `pyr`: the

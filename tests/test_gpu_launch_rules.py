@@ -42,3 +42,66 @@ def test_adjoint_items(w, h, tile, lpp, spec, occ, nd, det):
                              deterministic=det).cpu().numpy().astype(np.float64)
     assert np.abs(got - ref).max() <= 1e-4 * np.abs(ref).max()
     assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+# Brick builds read only the 16^3 blocks with an occupied brick, listed 256
+# at a time per CTA: no block, one voxel, a scattered quarter, every block,
+# and (n = 1024) more blocks per CTA than one list holds.
+@pytest.mark.parametrize("n,fill", [(16, "none"), (16, "one"), (32, "all"), (64, "some"),
+                                    (128, "one"), (256, "some"), (256, "none"), (1024, "some")])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("planned", [True, False])
+def test_brick_build_lists(n, fill, dtype, planned):
+    if n == 1024 and dtype == "f32":
+        pytest.skip("the binary16 case covers the lists of this size")
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    g = torch.zeros((n, n, n, 4), device="cuda")
+    if fill == "one":
+        g[n - 1, 0, n // 2, 3] = 0.5
+    elif fill == "all":
+        g.uniform_(0.1, 1.0, generator=gen)
+    elif fill == "some":  # one voxel in each of a quarter of the 16^3 blocks
+        m = n // 16
+        pick = torch.rand((m, m, m), device="cuda", generator=gen) < 0.25
+        z, y, x = pick.nonzero().mul(16).add(5).unbind(1)
+        g[z, y, x] = torch.rand((len(z), 4), device="cuda", generator=gen)
+    dense = vct.build_mips(g, dtype=dtype)
+    if planned:
+        bricks = vct.build_mips(g, dtype=dtype, layout="bricks")
+    else:
+        bricks = vct.Pyramid(n, dtype=dtype, layout="bricks",
+                             occupied=vct.plan_bricks(g, dtype=dtype)[0])
+        bricks.storage.fill_(255)  # nothing may be left from before
+        vct.build_mips(g, dtype=dtype, out=bricks)
+    if planned:
+        vct.pyramid_status(bricks)
+    for l in range(1 if n == 1024 else 0, dense.levels):
+        assert torch.equal(vct.read_level(dense, l), vct.read_level(bricks, l)), l
+
+
+def test_planned_build_checks_its_pool_and_scratch():
+    import ctypes
+    lib, abi = vct.lib(), vct._abi
+    g = torch.rand((64, 64, 64, 4), device="cuda")
+    occ, _ = vct.plan_bricks(g)
+    sb = lib.vct_pyramid_plan_scratch_bytes(64, 7, abi.VCT_F32)
+    scratch = torch.zeros(sb, dtype=torch.uint8, device="cuda")
+    at = ctypes.c_void_p(scratch.data_ptr())
+    stream = torch.cuda.current_stream().cuda_stream
+    assert lib.vct_pyramid_plan_bricks(ctypes.c_void_p(g.data_ptr()), 64, 7, abi.VCT_F32, at, sb,
+                                       None, None, stream) == abi.VCT_OK
+    small = vct.Pyramid(64, layout="bricks", occupied=occ - 1)
+    small.storage.zero_()
+    p = small.struct()
+    args = (ctypes.c_void_p(g.data_ptr()), ctypes.byref(p))
+    assert lib.vct_build_mips_planned(*args, at, sb - 1, stream) == abi.VCT_ERR_WORKSPACE
+    assert lib.vct_build_mips_planned(*args, None, sb, stream) == abi.VCT_ERR_WORKSPACE
+    assert lib.vct_build_mips_planned(*args, at, sb, stream) == abi.VCT_OK
+    with pytest.raises(vct.VctError) as e:
+        vct.pyramid_status(small)
+    assert e.value.status == abi.VCT_ERR_WORKSPACE
+    assert not vct.read_level(small, 0).any()
+    assert torch.allclose(vct.read_level(small, 6), g.mean(dim=(0, 1, 2)), rtol=1e-5)
+    d = vct.Pyramid(64).struct()
+    assert lib.vct_build_mips_planned(args[0], ctypes.byref(d), at, sb,
+                                      stream) == abi.VCT_ERR_INVALID_ARG
