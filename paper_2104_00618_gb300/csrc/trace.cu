@@ -395,12 +395,181 @@ __global__ void __launch_bounds__(kFwdThreads, kTraceMinBlocks) trace_kernel(con
   }
 }
 
+// Small launches: the warps of a group (L.group, 2 or 4) share a tile of 8 x 4
+// pixels, one pixel per lane, and split its cones: the first warp marches the
+// specular cone, the longest, the others the rest in turn (all of them,
+// without a specular cone).  Each warp leaves its part of D in shared memory
+// and the second warp sums the parts and writes the pixel.  The lanes of a
+// warp still march one cone in lock step.
+__device__ __forceinline__ void group_sync(int id, int threads) {
+  __syncwarp();  // (the barrier wants whole warps)
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+template <int DT, bool kVar, bool BR, bool AN>
+__global__ void __launch_bounds__(kFwdThreads, kTraceMinBlocks)
+    trace_split_kernel(const __grid_constant__ TraceLaunch L) {
+  constexpr int kWarps = kFwdThreads / 32;
+  uint32_t n_samp[3] = {0u, 0u, 0u}, n_cone[3] = {0u, 0u, 0u};
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int group = warp / L.group, q = warp % L.group;  // q: the warp's place in its group
+  const int bar = 1 + group, bar_threads = 32 * L.group;
+  const int n_cones = L.n_diffuse + L.spec_enable + L.occ_enable;
+  const float T0 = L.spec.t0_vox;
+  __shared__ uint2 s_lut[kSpreadLut];
+  __shared__ float4 s_part[kWarps][32];  // a warp's part of D; the specular warp's S
+  __shared__ float s_vis[kWarps][32];    // transmittance of the occlusion cone
+  __shared__ int s_item[kWarps];
+  extern __shared__ __align__(16) float4 s_tab[];
+  fill_step_table(s_tab, L.pyr, L.n_pyr, T0);
+  fill_spread_lut(s_lut);  // (its barrier also covers s_tab)
+
+  for (;;) {
+    if (q == 0 && lane == 0) s_item[group] = (int)atomicAdd(L.queue, 1u);
+    group_sync(bar, bar_threads);
+    const int item = s_item[group];
+    if (item >= L.total_tiles) break;  // (the whole group)
+    const int vi = find_view(L, item, false);
+    const DevView &V = L.views[vi];
+    const DevPyr &P = L.pyr[V.pyr];
+    const int t = item - V.tile_begin;
+    const int px = (t % V.tiles_x) * kSmallTileW + lane % kSmallTileW;
+    const int py = (t / V.tiles_x) * kSmallTileH + lane / kSmallTileW;
+    const bool inimg = px < V.W && py < V.H;
+    const int p = py * V.W + px;
+    const bool active = inimg && (V.mask == nullptr || V.mask[p] != 0);
+    float4 D = make_float4(0.f, 0.f, 0.f, 0.f);
+    float vis = 0.f;
+    if (active) {
+      float x[3], n[3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        x[a] = V.pos[3 * p + a];
+        n[a] = V.nrm[3 * p + a];
+      }
+      Apex A;
+      make_apex(P, x, n, L.normal_offset, A);
+      float Tf[3], Bf[3];
+      tangent_frame(n, Tf, Bf);
+      // warp 0: the specular cone; else every (group - 1)th of the others
+      const bool own_spec = L.spec_enable && q == 0;
+      const int step = own_spec ? n_cones : L.group - L.spec_enable;
+      for (int c = q; c < n_cones; c += step) {
+        const ConeSel cs = select_cone(c, L.spec_enable, L.occ_enable);
+        float w[3];
+        ConeConst cc;
+        const float4 *tab = nullptr;
+        if (cs.kind == kSpecular) {
+          reflect_dir(x, V.cam, n, w);
+          cc = spec_const(P, L.spec, V.rough, p);
+        } else if (cs.kind == kOcclusion) {
+          w[0] = L.light[0];
+          w[1] = L.light[1];
+          w[2] = L.light[2];
+          cc = P.occ;
+          tab = step_table(s_tab, V.pyr, 1);
+        } else {
+          const float *d = L.diffuse_dir[cs.diffuse_index];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) w[a] = fmaf(Tf[a], d[0], fmaf(Bf[a], d[1], n[a] * d[2]));
+          cc = P.diffuse;
+          tab = step_table(s_tab, V.pyr, 0);
+        }
+        int mode = kPlain;
+        if constexpr (kVar) {
+          if (cs.kind == kOcclusion && (L.var.flags & VCT_FLAG_OCC_SMOOTH)) mode = kOccSmooth;
+          if (cs.kind == kDiffuse && (L.var.flags & VCT_FLAG_DIFFUSE_FIRST_HIT)) mode = kFirstHit;
+        }
+        float trans;
+        uint2 cst;
+        float4 r = march<DT, kVar, BR, AN>(P, A, w, cc, T0, s_lut, tab, n_samp[cs.kind], trans,
+                                           cst, mode, &L.var);
+        n_cone[cs.kind] += 1u;
+        if (V.state) V.state[(size_t)c * V.W * V.H + p] = cst;
+        if (cs.kind == kDiffuse) {
+          const float wt = L.diffuse_weight[cs.diffuse_index];
+          D.x = fmaf(wt, r.x, D.x);
+          D.y = fmaf(wt, r.y, D.y);
+          D.z = fmaf(wt, r.z, D.z);
+          D.w = fmaf(wt, r.w, D.w);
+        } else if (cs.kind == kOcclusion) {
+          vis = trans;
+        } else {
+          if constexpr (kVar) {
+            if (L.var.flags & VCT_FLAG_SPEC_GRACE) {
+              const float f = spec_grace(L.var, w);
+              r.x *= f;
+              r.y *= f;
+              r.z *= f;
+            }
+          }
+          D = r;  // (this warp has no other cone)
+        }
+      }
+    }
+    s_part[warp][lane] = D;
+    s_vis[warp][lane] = vis;
+    group_sync(bar, bar_threads);
+    if (q == 1 && inimg) {
+      const int w0 = group * L.group;
+      float4 S = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (L.spec_enable) {
+        S = s_part[w0][lane];
+      } else {
+        const float4 o = s_part[w0][lane];
+        D.x += o.x;
+        D.y += o.y;
+        D.z += o.z;
+        D.w += o.w;
+        vis += s_vis[w0][lane];
+      }
+      for (int k = 2; k < L.group; ++k) {
+        const float4 o = s_part[w0 + k][lane];
+        D.x += o.x;
+        D.y += o.y;
+        D.z += o.z;
+        D.w += o.w;
+        vis += s_vis[w0 + k][lane];
+      }
+      if (!(L.occ_enable && active)) vis = 1.0f;
+      if (V.outD) reinterpret_cast<float4 *>(V.outD)[p] = D;
+      if (V.outS) reinterpret_cast<float4 *>(V.outS)[p] = S;
+      if (V.outV) V.outV[p] = vis;
+      if constexpr (kVar) {
+        if (V.outL) {
+          float4 Lp = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (active) Lp = shade_spec(L.var, V, p, S, shade_first(L.var, V, p, D, vis));
+          reinterpret_cast<float4 *>(V.outL)[p] = Lp;
+        }
+      }
+    }
+    // (the next item's barrier orders the parts' reads with their next writes)
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t ns = __reduce_add_sync(0xffffffffu, n_samp[k]);
+    const uint32_t nc = __reduce_add_sync(0xffffffffu, n_cone[k]);
+    if (lane == 0) {
+      if (ns) atomicAdd(L.stats + k, (unsigned long long)ns);
+      if (nc) atomicAdd(L.stats + 3 + k, (unsigned long long)nc);
+    }
+  }
+}
+
 // Dynamic shared memory of a launch: the step tables of its pyramids.
 inline size_t step_table_bytes(int n_pyr) { return (size_t)n_pyr * 2 * kStepTab * sizeof(float4); }
 
 template <int LPP, int DT, bool BR, bool AN = false>
 cudaError_t launch_t(const TraceLaunch &L, int grid, cudaStream_t s) {
   const size_t dyn = step_table_bytes(L.n_pyr);
+  if constexpr (LPP == 1) {
+    if (L.group) {
+      if (L.var.flags)
+        trace_split_kernel<DT, true, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
+      else
+        trace_split_kernel<DT, false, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
+      return cudaGetLastError();
+    }
+  }
   if (L.var.flags)
     trace_kernel<LPP, DT, true, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
   else

@@ -343,14 +343,60 @@ TuneKey tune_key(const vct_pyramid *pyrs, const vct_view *views, const vct_trace
                  views[0].roughness != nullptr, P->flags);
 }
 
-vct_launch_config default_cfg() { return vct_launch_config{16, 16, 1, 0}; }
+int64_t total_pixels(const vct_view *views, int32_t n_views) {
+  int64_t px = 0;
+  for (int i = 0; i < n_views; ++i) px += (int64_t)views[i].width * views[i].height;
+  return px;
+}
+
+// Tile of a launch that the caller gives no shape for.  Where the specular
+// aperture follows the roughness, a larger tile sorts more cones by length;
+// a smaller one leaves less idle in the last wave of warps.  Measured (9 + 1
+// + 1 cones, 256^3), 8 x 8 / 8 x 16 / 16 x 16: 230 K pixels 1077 / 1032 /
+// 1598 us, 0.92 M (mean of eight scenes) 3189 / 2994 / 3131, 1.05 M 3532 /
+// 3312 / 3274, 2.07 M 7201 / 6785 / 6702 (binary16, bricks, shaded and
+// anisotropic alike); one aperture (6 + 1 cones, 64^3): 0.52 M 661 / 659 /
+// 844, 2.07 M 2393 / 2430 / 2539.
+vct_launch_config default_cfg(const vct_view *views, int32_t n_views, const vct_trace_params &P) {
+  bool rough = false;
+  for (int i = 0; i < n_views; ++i) rough |= views[i].roughness != nullptr;
+  if (!P.spec_enable || !rough || P.spec_aperture_min == P.spec_aperture_max)
+    return vct_launch_config{8, 8, 1, 0};
+  if (total_pixels(views, n_views) < 1000000) return vct_launch_config{8, 16, 1, 0};
+  return vct_launch_config{16, 16, 1, 0};
+}
 
 vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs,
-                           const vct_view *views, const vct_trace_params *P) {
+                           const vct_view *views, int32_t n_views, const vct_trace_params *P,
+                           bool &tuned) {
+  tuned = false;
   if (cfg) return *cfg;
   std::lock_guard<std::mutex> g(g_tune_mu);
   auto it = g_tuned.find(tune_key(pyrs, views, P));
-  return it == g_tuned.end() ? default_cfg() : it->second;
+  tuned = it != g_tuned.end();
+  return tuned ? it->second : default_cfg(views, n_views, *P);
+}
+
+// Warps that share a tile's cones in a launch whose shape is the library's
+// choice, or 0 (each warp takes whole tiles).  A warp that marches all cones
+// of its 32 pixels in series takes the same time however few pixels there
+// are, so the cones of a launch of few warps are split: four ways while its
+// warps are then no more than the chip holds at once, two ways up to four
+// times that.  Measured, split 4 / 2 / 1 ways: 9 + 1 + 1 cones at 256^3, 5917
+// pixels 141 / 210 / 318 us, 16 384: 173 / 204 / 304, 25 600: 240 / 252 / 299,
+// 57 600: 396 / 399 / 407, 129 600: 758 / 689 / 695, 230 400 (the last in 8 x
+// 16 tiles): 1271 / 1135 / 1032; 6 + 1 cones at 64^3, 16 384: 73 / 75 / 107,
+// 57 600: 142 / 121 / 144, 129 600: 269 / 210 / 229.
+int trace_group(const vct_view *views, int32_t n_views, const vct_trace_params &P, int sms) {
+  const int others = P.n_diffuse + P.occ_enable;
+  if (others + P.spec_enable < 2) return 0;
+  int64_t tiles = 0;
+  for (int i = 0; i < n_views; ++i)
+    tiles += (int64_t)((views[i].width + kSmallTileW - 1) / kSmallTileW) *
+             ((views[i].height + kSmallTileH - 1) / kSmallTileH);
+  const int64_t warps = (int64_t)sms * kTraceMinBlocks * (kFwdThreads / 32);
+  if (tiles * 4 <= warps && others >= 3) return 4;
+  return tiles * 2 <= warps * 4 ? 2 : 0;
 }
 
 struct TraceStatsLayout {
@@ -570,7 +616,7 @@ size_t vct_trace_workspace_bytes(void) { return 256; }
 
 static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_view *views,
                              int32_t n_views, const vct_trace_params *params,
-                             const vct_launch_config &cfg, void *workspace,
+                             const vct_launch_config &shape, bool any_shape, void *workspace,
                              size_t workspace_bytes, cudaStream_t stream, bool zero_stats) {
   auto L = std::make_unique<TraceLaunch>();
   memset(L.get(), 0, sizeof(TraceLaunch));
@@ -581,6 +627,12 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
     if (st != VCT_OK) return st;
   }
   L->n_pyr = n_pyr;
+  const int sms = sm_count();
+  vct_launch_config cfg = shape;
+  if (any_shape) {
+    L->group = trace_group(views, n_views, *params, sms);
+    if (L->group) cfg = vct_launch_config{kSmallTileW, kSmallTileH, 1, 0};
+  }
   L->tile_w = cfg.tile_w;
   L->tile_h = cfg.tile_h;
   uint8_t *ws = static_cast<uint8_t *>(workspace);
@@ -592,7 +644,6 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
   int per_sm = cfg.ctas_per_sm;
   if (per_sm == 0)
     per_sm = std::max(1, trace_occupancy(cfg.lanes_per_pixel, pyrs[0].dtype, params->flags != 0));
-  const int sms = sm_count();
   for (int v0 = 0; v0 < n_views; v0 += kMaxViewsPerLaunch) {
     const int nv = std::min(kMaxViewsPerLaunch, n_views - v0);
     int cursor = 0;
@@ -609,10 +660,16 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
                   "vct_trace: views of one call must use pyramids of one dtype, and all or "
                   "none anisotropic");
     L->n_views = nv;
-    const int grid = std::max(1, std::min(cursor, per_sm * sms));
+    int grid = std::max(1, std::min(cursor, per_sm * sms));
     // about two waves of the launch's warps, in small tiles, at the end
     const int64_t tail_px = (int64_t)2 * grid * (kFwdThreads / 32) * kSmallTileW * kSmallTileH;
-    L->total_tiles = assign_tail_tiles(L->views, nv, cfg.tile_w, cfg.tile_h, tail_px, L->n_big);
+    if (L->group) {
+      L->total_tiles = L->n_big = cursor;
+      const int per_cta = kFwdThreads / 32 / L->group;  // tiles a CTA takes at a time
+      grid = std::min(grid, (cursor + per_cta - 1) / per_cta);
+    } else {
+      L->total_tiles = assign_tail_tiles(L->views, nv, cfg.tile_w, cfg.tile_h, tail_px, L->n_big);
+    }
     if (v0 > 0 && (e = cudaMemsetAsync(L->queue, 0, 4, stream)) != cudaSuccess)
       return cuda_fail(e, "vct_trace queue clear");
     e = launch_trace(*L, cfg.lanes_per_pixel, pyrs[views[v0].pyramid].dtype, bricks, grid,
@@ -648,10 +705,11 @@ vct_status vct_trace(const vct_pyramid *pyrs, int32_t n_pyr, const vct_view *vie
                      vct_stream_t stream) {
   vct_status st = trace_checks(pyrs, n_pyr, views, n_views, params, workspace, workspace_bytes);
   if (st != VCT_OK) return st;
-  const vct_launch_config c = pick_cfg(cfg, pyrs, views, params);
+  bool tuned = false;
+  const vct_launch_config c = pick_cfg(cfg, pyrs, views, n_views, params, tuned);
   if (!cfg_ok(c)) return fail(VCT_ERR_INVALID_ARG, "vct_trace: bad launch config");
-  return trace_impl(pyrs, n_pyr, views, n_views, params, c, workspace, workspace_bytes,
-                    (cudaStream_t)stream, true);
+  return trace_impl(pyrs, n_pyr, views, n_views, params, c, cfg == nullptr && !tuned, workspace,
+                    workspace_bytes, (cudaStream_t)stream, true);
 }
 
 vct_status vct_autotune_trace(const vct_pyramid *pyrs, int32_t n_pyr, const vct_view *views,
@@ -667,14 +725,15 @@ vct_status vct_autotune_trace(const vct_pyramid *pyrs, int32_t n_pyr, const vct_
   const int tiles[4][2] = {{4, 8}, {8, 8}, {8, 16}, {16, 16}};
   const int lpps[4] = {1, 2, 4, 8};
   float best_ms = 1e30f;
-  vct_launch_config bc = default_cfg();
+  vct_launch_config bc{16, 16, 1, 0};
   for (auto &t : tiles)
     for (int lpp : lpps) {
       vct_launch_config c{t[0], t[1], lpp, 0};
       float ms_sum = 0.f;
       for (int rep = 0; rep < 3; ++rep) {
         cudaEventRecord(e0, s);
-        st = trace_impl(pyrs, n_pyr, views, n_views, params, c, workspace, workspace_bytes, s, true);
+        st = trace_impl(pyrs, n_pyr, views, n_views, params, c, false, workspace, workspace_bytes, s,
+                        true);
         cudaEventRecord(e1, s);
         if (st != VCT_OK) break;
         if (cudaEventSynchronize(e1) != cudaSuccess) {
@@ -766,8 +825,7 @@ vct_status trace_backward_impl(const vct_pyramid *pyr, const vct_view *views,
   const int sms = sm_count();
   // Warps of a full chip (two CTAs of 256 threads per SM).
   const int64_t resident = (int64_t)sms * 2 * (kTraceThreads / 32);
-  int64_t pixels = 0;
-  for (int i = 0; i < n_views; ++i) pixels += (int64_t)views[i].width * views[i].height;
+  const int64_t pixels = total_pixels(views, n_views);
   // Tiles of 8 x 8 pixels; of 8 x 4, one round of a warp, where even those
   // are fewer than half the warps of a full chip (all of them for the
   // reproducible mode, whose rounds cost more).  Measured on a 64^3 grid

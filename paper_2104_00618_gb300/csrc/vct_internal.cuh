@@ -316,7 +316,8 @@ struct TraceLaunch {
   int n_views, total_tiles, tile_w, tile_h;
   int n_big;  // items [0, n_big) are big tiles, the rest small tiles
   int n_pyr;  // pyramids in pyr[]
-  int n_diffuse, spec_enable, occ_enable, pad0;
+  int n_diffuse, spec_enable, occ_enable;
+  int group;  // warps that share a tile's cones (small launches), or 0
   Variants var;
   float diffuse_dir[VCT_MAX_DIFFUSE][3];
   float diffuse_weight[VCT_MAX_DIFFUSE];

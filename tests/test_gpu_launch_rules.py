@@ -105,3 +105,45 @@ def test_planned_build_checks_its_pool_and_scratch():
     d = vct.Pyramid(64).struct()
     assert lib.vct_build_mips_planned(args[0], ctypes.byref(d), at, sb,
                                       stream) == abi.VCT_ERR_INVALID_ARG
+
+
+# A launch without a shape shares a tile's cones among 4 warps (up to 608
+# tiles of 8 x 4 pixels on 152 SMs), 2 (up to 4864) or none, where the tile
+# depends on the roughness; each against one warp per 8 x 8 tile: the cones
+# march the same steps (states bit for bit), D sums the same cones in another
+# order (at most 32 terms, 2^-24 each).
+@pytest.mark.parametrize("w,h,spec,occ,nd,rough", [
+    (1, 1, 1, 1, 6, False), (9, 5, 0, 1, 1, False), (37, 21, 1, 0, 2, True), (64, 33, 0, 0, 5, False),
+    (160, 121, 1, 1, 6, True), (160, 125, 1, 1, 6, True), (400, 389, 1, 1, 1, False),
+    (400, 393, 1, 1, 1, False), (500, 400, 1, 0, 1, True), (300, 200, 1, 0, 0, True)])
+@pytest.mark.parametrize("dtype,layout,flags", [("f32", "dense", 0), ("f16", "bricks", 0),
+                                                ("f32", "aniso", 0), ("f32", "dense", 15),
+                                                ("f32", "dense", 32 + 24)])
+def test_forward_shapes(w, h, spec, occ, nd, rough, dtype, layout, flags):
+    n = 16
+    rng = np.random.default_rng(w + h)
+    scene = vs.box_scene(n, 4, 5, room=True)
+    view = vs.interior_view(scene, w, h, rng, with_roughness=rough)
+    view["mask"] = (rng.random(w * h) >= 0.1).astype(np.uint8)
+    dirs, wts = vs.cone_table_ring6()
+    prm = vs.trace_params(dirs[:nd], wts[:nd], 1.0, spec_enable=spec, spec_aperture_min=0.3,
+                          spec_aperture_max=0.9, occ_enable=occ, light=scene["light"])
+    prm = vs.variant_params(prm, flags)
+    P = vct.build_mips(torch.from_numpy(scene["grid"]).cuda(), dtype=dtype, layout=layout)
+    out = []
+    for cfg in (None, vct.launch_config(8, 8, 1)):
+        v = vct.View.from_host(view)
+        if flags & vct.FLAG_SHADE:
+            v.albedo = torch.full((w * h, 3), 0.7, device="cuda")
+            v.alloc_outputs(radiance=True)
+        v.alloc_cone_state(prm).cone_state.zero_()
+        stats = vct.read_stats(vct.trace(P, v, prm, cfg=cfg))
+        out.append((v, stats))
+    (a, sa), (b, sb) = out
+    assert sa == sb
+    assert torch.equal(a.cone_state, b.cone_state)
+    assert torch.equal(a.out_specular, b.out_specular)
+    assert torch.equal(a.out_visibility, b.out_visibility)
+    for x, y in ((a.out_diffuse, b.out_diffuse), (a.out_radiance, b.out_radiance)):
+        if x is not None:
+            assert (x - y).abs().max() <= 32 * 2.0 ** -24 * max(1.0, float(y.abs().max()))
