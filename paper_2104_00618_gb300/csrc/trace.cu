@@ -406,9 +406,9 @@ __device__ __forceinline__ void group_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 template <int DT, bool kVar, bool BR, bool AN>
-__global__ void __launch_bounds__(kFwdThreads, kTraceMinBlocks)
+__global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
     trace_split_kernel(const __grid_constant__ TraceLaunch L) {
-  constexpr int kWarps = kFwdThreads / 32;
+  constexpr int kWarps = kSplitThreads / 32;
   uint32_t n_samp[3] = {0u, 0u, 0u}, n_cone[3] = {0u, 0u, 0u};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int group = warp / L.group, q = warp % L.group;  // q: the warp's place in its group
@@ -564,9 +564,9 @@ cudaError_t launch_t(const TraceLaunch &L, int grid, cudaStream_t s) {
   if constexpr (LPP == 1) {
     if (L.group) {
       if (L.var.flags)
-        trace_split_kernel<DT, true, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
+        trace_split_kernel<DT, true, BR, AN><<<grid, kSplitThreads, dyn, s>>>(L);
       else
-        trace_split_kernel<DT, false, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
+        trace_split_kernel<DT, false, BR, AN><<<grid, kSplitThreads, dyn, s>>>(L);
       return cudaGetLastError();
     }
   }

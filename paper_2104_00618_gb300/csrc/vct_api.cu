@@ -352,17 +352,17 @@ int64_t total_pixels(const vct_view *views, int32_t n_views) {
 // Tile of a launch that the caller gives no shape for.  Where the specular
 // aperture follows the roughness, a larger tile sorts more cones by length;
 // a smaller one leaves less idle in the last wave of warps.  Measured (9 + 1
-// + 1 cones, 256^3), 8 x 8 / 8 x 16 / 16 x 16: 230 K pixels 1077 / 1032 /
-// 1598 us, 0.92 M (mean of eight scenes) 3189 / 2994 / 3131, 1.05 M 3532 /
-// 3312 / 3274, 2.07 M 7201 / 6785 / 6702 (binary16, bricks, shaded and
-// anisotropic alike); one aperture (6 + 1 cones, 64^3): 0.52 M 661 / 659 /
-// 844, 2.07 M 2393 / 2430 / 2539.
+// + 1 cones, 256^3), 8 x 8 / 8 x 16 / 16 x 16: 0.41 M pixels 1671 / 1598 / 2049
+// us, 0.92 M 3307 / 3175 / 3631, 2.07 M 7153 / 6649 / 6880, 3.69 M 12467 /
+// 11544 / 11082 (binary16, bricks, shaded and anisotropic alike within a
+// tenth of that line); one aperture (6 + 1 cones, 64^3): 0.52 M 656 / 704 /
+// 804, 2.07 M 2373 / 2398 / 2596.
 vct_launch_config default_cfg(const vct_view *views, int32_t n_views, const vct_trace_params &P) {
   bool rough = false;
   for (int i = 0; i < n_views; ++i) rough |= views[i].roughness != nullptr;
   if (!P.spec_enable || !rough || P.spec_aperture_min == P.spec_aperture_max)
     return vct_launch_config{8, 8, 1, 0};
-  if (total_pixels(views, n_views) < 1000000) return vct_launch_config{8, 16, 1, 0};
+  if (total_pixels(views, n_views) < 2500000) return vct_launch_config{8, 16, 1, 0};
   return vct_launch_config{16, 16, 1, 0};
 }
 
@@ -394,7 +394,7 @@ int trace_group(const vct_view *views, int32_t n_views, const vct_trace_params &
   for (int i = 0; i < n_views; ++i)
     tiles += (int64_t)((views[i].width + kSmallTileW - 1) / kSmallTileW) *
              ((views[i].height + kSmallTileH - 1) / kSmallTileH);
-  const int64_t warps = (int64_t)sms * kTraceMinBlocks * (kFwdThreads / 32);
+  const int64_t warps = (int64_t)sms * kSplitBlocks * (kSplitThreads / 32);
   if (tiles * 4 <= warps && others >= 3) return 4;
   return tiles * 2 <= warps * 4 ? 2 : 0;
 }
@@ -665,8 +665,8 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
     const int64_t tail_px = (int64_t)2 * grid * (kFwdThreads / 32) * kSmallTileW * kSmallTileH;
     if (L->group) {
       L->total_tiles = L->n_big = cursor;
-      const int per_cta = kFwdThreads / 32 / L->group;  // tiles a CTA takes at a time
-      grid = std::min(grid, (cursor + per_cta - 1) / per_cta);
+      const int per_cta = kSplitThreads / 32 / L->group;  // tiles a CTA takes at a time
+      grid = std::max(1, std::min((cursor + per_cta - 1) / per_cta, kSplitBlocks * sms));
     } else {
       L->total_tiles = assign_tail_tiles(L->views, nv, cfg.tile_w, cfg.tile_h, tail_px, L->n_big);
     }
