@@ -21,10 +21,11 @@ struct TableArgs {
 // One warp per level-0 brick: where any channel of its 512 texels is
 // non-zero, the brick and the bricks above it in every bricked level are
 // flagged (the flags start at 0; warps that share a coarser brick store the
-// same 1).  level0 is dense [z][y][x][4]; the brick's rows of 8 texels are 128
+// same 1); `small`: each level-0 flag is written, 0 or 1, and no other.  level0 is dense [z][y][x][4]; the brick's rows of 8 texels are 128
 // bytes.  512^3: 0.32 ms for 2.15 GB, the HBM copy rate.
 __global__ void __launch_bounds__(256) occupancy_kernel(const float4 *level0, int n,
-                                                        const __grid_constant__ TableArgs a) {
+                                                        const __grid_constant__ TableArgs a,
+                                                        bool small) {
   const int lane = threadIdx.x & 31;
   const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -39,13 +40,17 @@ __global__ void __launch_bounds__(256) occupancy_kernel(const float4 *level0, in
       any |= (v.x != 0.0f) | (v.y != 0.0f) | (v.z != 0.0f) | (v.w != 0.0f);
     }
     any = __any_sync(0xffffffffu, any);
-    if (any && lane < a.nbricked) a.tbl[lane][id >> (3 * lane)] = 1u;
+    if (small) {
+      if (lane == 0) a.tbl[0][id] = any ? 1u : 0u;
+    } else if (any && lane < a.nbricked) {
+      a.tbl[lane][id >> (3 * lane)] = 1u;
+    }
   }
 }
 
 // Flags -> slots, by an exclusive scan over all bricked levels in level order:
-// the tables are contiguous, with zeros in the gaps between them, so they are
-// scanned as one array.  kScanCtas CTAs take a part each; count_kernel leaves
+// the tables follow one another without gaps (a level of 64 bricks or more
+// fills 256-byte lines, the last one has 8), so they are scanned as one array.  kScanCtas CTAs take a part each; count_kernel leaves
 // the parts' sums in the header's free words, slots_kernel adds those before
 // its own.  At 512^3 (300 K flags) one CTA alone took 232 us with one flag per
 // thread and pass, 69 us with 16 (its SM's share of the L2 bandwidth).
@@ -56,8 +61,9 @@ constexpr int kScanPass = kScanThreads * kScanRun;
 static_assert(16 + 4 * kScanCtas <= kHeaderBytes, "the parts' sums lie in the header");
 
 struct ScanArgs {
-  uint32_t *flags, *sums;
+  uint32_t *flags, *sums;  // sums: null where one pass of one CTA holds every flag
   uint64_t words, part;  // part: words per CTA, a multiple of kScanPass
+  uint64_t bricks0;      // level 0's
   uint32_t *status;
   unsigned long long *count;
   uint64_t capacity;
@@ -93,12 +99,29 @@ __global__ void __launch_bounds__(kScanThreads) slots_kernel(const __grid_consta
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   // (every warp sums the parts; kScanCtas <= 64)
   uint32_t before_part = 0u, total = 0u;
-  for (int i = lane; i < (int)gridDim.x; i += 32) {
+  for (int i = lane; a.sums != nullptr && i < (int)gridDim.x; i += 32) {
     const uint32_t c = a.sums[i];
     total += c;
     if (i < (int)blockIdx.x) before_part += c;
   }
   total = __reduce_add_sync(0xffffffffu, total);
+  if (a.sums == nullptr) {  // one part of one pass: the coarser flags and the count here
+    const uint32_t *child = a.flags;
+    for (uint64_t nb = a.bricks0 >> 3, at = a.bricks0; nb >= 8; at += nb, nb >>= 3) {
+      for (uint64_t p = threadIdx.x; p < nb; p += blockDim.x) {
+        const uint4 u = *reinterpret_cast<const uint4 *>(child + 8 * p);
+        const uint4 v = *reinterpret_cast<const uint4 *>(child + 8 * p + 4);
+        if (at + p < a.words) a.flags[at + p] = u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w;
+      }
+      child = a.flags + at;
+      __syncthreads();
+    }
+    const uint64_t e = (uint64_t)threadIdx.x * kScanRun;
+    const uint32_t c = __reduce_add_sync(0xffffffffu, __popc(load_flags(a, e, a.words)));
+    if (lane == 0) s_warp[1][wid] = c;
+    __syncthreads();
+    total = __reduce_add_sync(0xffffffffu, s_warp[1][lane]);
+  }
   uint32_t run = 1u + __reduce_add_sync(0xffffffffu, before_part);  // next slot of this part
   const bool fits = 1ull + total <= a.capacity;  // else: leave every brick empty, report it
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -185,11 +208,10 @@ cudaError_t launch_brick_tables(const float *level0, int n, int levels, const La
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // the tables are contiguous, each rounded up to 256 bytes
   uint8_t *first = reinterpret_cast<uint8_t *>(a.tbl[0]);
   const int last = a.nbricked - 1;
   const uint64_t bytes =
-      (uint64_t)(reinterpret_cast<uint8_t *>(a.tbl[last]) - first) + align256(a.nb[last] * 4);
+      (uint64_t)(reinterpret_cast<uint8_t *>(a.tbl[last]) - first) + a.nb[last] * 4;
   if (planned != nullptr) {
     const uint64_t words = bytes / 16;
     const int grid = (int)std::min<uint64_t>((words + 255) / 256, (uint64_t)sms * 4);
@@ -199,11 +221,14 @@ cudaError_t launch_brick_tables(const float *level0, int n, int levels, const La
         reinterpret_cast<const unsigned long long *>(planned + kHeaderCountOff));
     return cudaGetLastError();
   }
-  cudaError_t e = cudaMemsetAsync(first, 0, bytes, s);
+  // A grid whose flags one pass of one CTA holds (n <= 128) needs two launches.
+  const bool small = bytes / 4 <= (uint64_t)kScanPass;
+  cudaError_t e = small ? cudaSuccess : cudaMemsetAsync(first, 0, bytes, s);
   if (e != cudaSuccess) return e;
   const uint64_t warps = a.nb[0];
   const int grid = (int)std::min<uint64_t>((warps + 7) / 8, (uint64_t)sms * 16);
-  occupancy_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4 *>(level0), n, a);
+  occupancy_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4 *>(level0), n, a,
+                                        small);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   ScanArgs c{};
   c.flags = reinterpret_cast<uint32_t *>(first);
@@ -215,8 +240,13 @@ cudaError_t launch_brick_tables(const float *level0, int n, int levels, const La
   c.count = a.count;
   c.capacity = capacity;
   const int parts = (int)((c.words + c.part - 1) / c.part);
-  count_kernel<<<parts, kScanThreads, 0, s>>>(c);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  c.bricks0 = a.nb[0];
+  if (small) {
+    c.sums = nullptr;
+  } else {
+    count_kernel<<<parts, kScanThreads, 0, s>>>(c);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   slots_kernel<<<parts, kScanThreads, 0, s>>>(c);
   return cudaGetLastError();
 }

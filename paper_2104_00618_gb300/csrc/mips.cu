@@ -381,17 +381,19 @@ __device__ __forceinline__ void wait_for_previous_grid() {
 }
 
 // Levels 0 .. top (top <= 4) of one patch of X x 16 x 16 level-0 voxels per
-// CTA (X = min(n, 256); the patch's origin a multiple of its extent), so
+// CTA (16 <= X <= 256; the patch's origin a multiple of its extent), so
 // that the levels above 1 are reduced on chip instead of re-reading level 1.
 // The patch is taken in 16 phases, one per level-2 row (qy, qz) of it, each
 // phase the four level-1 rows (2 qy + iy, 2 qz + iz), in units of 8 x 4
 // level-1 cells: lane = cx' | row << 3 (row = iy | iz << 1), so a unit holds
 // four whole level-2 cells and a warp reduces them with shuffles, with no
-// barrier between phases.  Warp w takes units w and w + 8 of each phase.  A
+// barrier between phases.  The CTA takes 16 units at a time, warp w the w-th
+// and the w+8-th: one phase where X = 256, several phases' where X is smaller.
+// A
 // lane's cell: its 8 children as four 32-byte x pairs (rows of a unit are
 // 256-byte pieces), written to level 0 at Morton codes 8 code .. 8 code + 7
 // (child jx | jy << 1 | jz << 2, the x pairs contiguous), and their mean to
-// level 1.  The loads of the next phase are issued as soon as the stores have
+// level 1.  The next 16 units' loads are issued as soon as the stores have
 // taken the registers.  After the 16 phases the patch's level-3 and level-4
 // texels come from its level-2 values, kept in shared memory.  Level-1 means
 // add the children in the order the TMA pack kernel does for the same cell
@@ -419,7 +421,7 @@ template <int DT>
 __device__ __forceinline__ typename Tex<DT>::T *level_ptr(const StreamArgs &a, int l) {
   return reinterpret_cast<typename Tex<DT>::T *>(a.lvl[l]);
 }
-template <int DT>
+template <int DT, bool kWide>
 __global__ void __launch_bounds__(256, 2) stream_levels_kernel(const __grid_constant__ StreamArgs a) {
   __shared__ float4 s2[16 * (kPatchX / 4)];  // the patch's level 2, row qz * 4 + qy
   __shared__ float4 s3[4 * (kPatchX / 8)];   // level 3, row rz * 2 + ry
@@ -428,24 +430,36 @@ __global__ void __launch_bounds__(256, 2) stream_levels_kernel(const __grid_cons
   const uint32_t pxn = n / X, pyn = n / kPatchYZ;
   const uint64_t patches = (uint64_t)pxn * pyn * pyn;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t units = hx / 8;  // units per phase (2 .. 16)
+  const uint32_t units = hx / 8;  // units per phase (1 .. 16)
   const uint32_t row = lane >> 3;
   float4 r[2][8];
-  // level-1 cell (gx, gy, gz) of this lane in unit slot k of phase p of patch P
-  auto cell = [&](uint64_t P, int p, int k, uint32_t &gx, uint32_t &gy, uint32_t &gz) {
-    const uint32_t u = warp + 8u * (uint32_t)k;
+  // Phase and unit of this warp's slot k of step it.  kWide: 16 units per
+  // phase, a step is a phase.
+  const uint32_t ushift = 31u - (uint32_t)__clz((int)units);  // (a power of two)
+  auto phase_of = [&](int it, int k) {
+    return kWide ? it : (int)((16u * (uint32_t)it + warp + 8u * (uint32_t)k) >> ushift);
+  };
+  auto unit_of = [&](int it, int k) {
+    return kWide ? warp + 8u * (uint32_t)k
+                 : (16u * (uint32_t)it + warp + 8u * (uint32_t)k) & (units - 1u);
+  };
+  const int steps = kWide ? 16 : (int)units;
+  // level-1 cell (gx, gy, gz) of this lane in slot k of step it of patch P
+  auto cell = [&](uint64_t P, int it, int k, uint32_t &gx, uint32_t &gy, uint32_t &gz) {
+    const int p = phase_of(it, k);
+    const uint32_t u = unit_of(it, k);
     const uint32_t px = (uint32_t)(P % pxn), py = (uint32_t)((P / pxn) % pyn),
                    pz = (uint32_t)(P / ((uint64_t)pxn * pyn));
     gx = px * hx + 8u * u + (lane & 7u);
     gy = py * (kPatchYZ / 2) + 2u * (uint32_t)(p & 3) + (row & 1u);
     gz = pz * (kPatchYZ / 2) + 2u * (uint32_t)(p >> 2) + (row >> 1);
-    return u < units;
+    return !kWide || u < units;
   };
-  auto load = [&](uint64_t P, int p) {
+  auto load = [&](uint64_t P, int it) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       uint32_t gx, gy, gz;
-      if (!cell(P, p, k, gx, gy, gz)) continue;
+      if (!cell(P, it, k, gx, gy, gz)) continue;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {  // q = jy | jz << 1
         const uint64_t y = 2 * gy + (q & 1), z = 2 * gz + (q >> 1);
@@ -457,13 +471,13 @@ __global__ void __launch_bounds__(256, 2) stream_levels_kernel(const __grid_cons
   for (uint64_t P = blockIdx.x; P < patches; P += gridDim.x) {
     const uint32_t px = (uint32_t)(P % pxn), py = (uint32_t)((P / pxn) % pyn),
                    pz = (uint32_t)(P / ((uint64_t)pxn * pyn));
-    for (int p = 0; p < 16; ++p) {
+    for (int it = 0; it < steps; ++it) {
       float4 m[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         uint32_t gx, gy, gz;
         m[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (!cell(P, p, k, gx, gy, gz)) continue;
+        if (!cell(P, it, k, gx, gy, gz)) continue;
         const uint32_t code = morton3(gx, gy, gz);
         if (in_bounds(8 * (uint64_t)code + 7, a.texels[0], kOobMip)) {
           if constexpr (DT == VCT_F32) {
@@ -494,9 +508,9 @@ __global__ void __launch_bounds__(256, 2) stream_levels_kernel(const __grid_cons
         m[k] = mul4(sum, 0.125f);
         if (in_bounds(code, a.texels[1], kOobMip)) st_texel(level_ptr<DT>(a, 1) + code, m[k]);
       }
-      // the next phase's loads (the stores above have taken r)
-      if (p + 1 < 16)
-        load(P, p + 1);
+      // the next step's loads (the stores above have taken r)
+      if (it + 1 < steps)
+        load(P, it + 1);
       else if (P + gridDim.x < patches)
         load(P + gridDim.x, 0);
       if (a.top < 2) continue;
@@ -504,8 +518,9 @@ __global__ void __launch_bounds__(256, 2) stream_levels_kernel(const __grid_cons
       // i at lane 2c + (i & 1) + (i >> 1) * 8 (child order, as mean8)
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const uint32_t u = warp + 8u * (uint32_t)k;
-        if (u >= units) continue;  // warp-uniform
+        const uint32_t u = unit_of(it, k);
+        if (kWide && u >= units) continue;  // warp-uniform
+        const int p = phase_of(it, k);
         const uint32_t c = lane & 3u;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -1127,7 +1142,14 @@ static cudaError_t build_dense_streamed(const float *level0, const vct_pyramid &
   StreamArgs sa{};
   sa.dense = reinterpret_cast<const float4 *>(level0);
   sa.n = pyr.n;
+  // The longest patches that still give every SM one: small grids are bound
+  // by the latency of a patch's steps (32^3 14.9 -> 7.8 us, 64^3 19.0 -> 8.7,
+  // 128^3 31.0 -> 18.7, binary16 23.0 -> 12.9, the levels above included).
+  auto patches_of = [&](int X) {
+    return (uint64_t)(pyr.n / X) * (pyr.n / kPatchYZ) * (pyr.n / kPatchYZ);
+  };
   sa.X = std::min(pyr.n, kPatchX);
+  while (sa.X > 16 && patches_of(sa.X) < (uint64_t)sms) sa.X /= 2;
   sa.top = std::min(kStreamTop, pyr.levels - 1);
   for (int l = 0; l <= sa.top; ++l) {
     sa.lvl[l] = base + L.level_off[l];
@@ -1135,12 +1157,12 @@ static cudaError_t build_dense_streamed(const float *level0, const vct_pyramid &
   }
   const bool tail = sa.top < pyr.levels - 1;
   sa.staging = (f16 && tail) ? reinterpret_cast<float4 *>(base + L.staging_off[0]) : nullptr;
-  const uint64_t patches = (uint64_t)(pyr.n / sa.X) * (pyr.n / kPatchYZ) * (pyr.n / kPatchYZ);
-  const int grid1 = (int)std::min<uint64_t>(patches, (uint64_t)sms * 2);
-  if (f16)
-    stream_levels_kernel<VCT_F16><<<grid1, 256, 0, s>>>(sa);
-  else
-    stream_levels_kernel<VCT_F32><<<grid1, 256, 0, s>>>(sa);
+  const int grid1 = (int)std::min<uint64_t>(patches_of(sa.X), (uint64_t)sms * 2);
+  auto kernel = sa.X == kPatchX ? (f16 ? stream_levels_kernel<VCT_F16, true>
+                                       : stream_levels_kernel<VCT_F32, true>)
+                                : (f16 ? stream_levels_kernel<VCT_F16, false>
+                                       : stream_levels_kernel<VCT_F32, false>);
+  kernel<<<grid1, 256, 0, s>>>(sa);
   cudaError_t e = cudaGetLastError();
   int m = sa.top;  // the last level made so far
   if (e != cudaSuccess || !tail) return e;
