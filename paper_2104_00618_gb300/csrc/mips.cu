@@ -681,6 +681,41 @@ __global__ void __launch_bounds__(1024) mip_tail_kernel(const TailArgs a) {
   }
 }
 
+// Levels m_top+1 .. m_top+k (k <= kGroupLevels) from the FP32 values of level
+// m_top, one CTA per 8^k of its texels, and the FP32 values of level m_top+k
+// to ping[0]: what comes before the one-CTA tail where level m_top holds more
+// than a CTA's worth (binary16 and brick pyramids, n >= 512).
+template <int DT, bool BR>
+__global__ void __launch_bounds__(256) mip_staged_group_kernel(const TailArgs a, int k) {
+  __shared__ float4 sm[512 + 64 + 8 + 1];
+  const int first = 1 << (3 * (k - 1));  // texels of level m_top+1 per CTA (<= 512)
+  const uint32_t g = blockIdx.x;
+  for (int j = threadIdx.x; j < first; j += blockDim.x) {
+    float4 ch[8];
+    const float4 *src = a.src0 + 8 * ((size_t)g * first + j);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) ch[q] = src[q];
+    const float4 v = mean8(ch);
+    put<DT, BR>(a.lvl, a.pool, a.bricked, a.pool_slots, a.n, a.m_top + 1, g * first + j, v);
+    sm[j] = v;
+  }
+  const float4 *cur = sm;
+  int cnt = first;
+  for (int l = 2; l <= k; ++l) {
+    __syncthreads();
+    float4 *nxt = const_cast<float4 *>(cur) + cnt;
+    const int nc = cnt / 8;
+    for (int j = threadIdx.x; j < nc; j += blockDim.x) {
+      const float4 v = mean8(cur + 8 * j);
+      put<DT, BR>(a.lvl, a.pool, a.bricked, a.pool_slots, a.n, a.m_top + l, g * nc + j, v);
+      nxt[j] = v;
+    }
+    cur = nxt;
+    cnt = nc;
+  }
+  if (threadIdx.x == 0) a.ping[0][g] = cur[0];  // (the thread that made it)
+}
+
 // Level to dense; `tbl` (bricked level) maps bricks to pool slots, else null.
 template <int DT>
 __global__ void read_level_kernel(const uint8_t *lvl, const uint32_t *tbl, const uint8_t *pool,
@@ -1064,6 +1099,25 @@ cudaError_t pack_t(const CUtensorMap &map, const PackArgs &a, int blocks, size_t
   return cudaGetLastError();
 }
 
+// The levels above m_top of a pyramid whose level m_top has FP32 values in
+// staging (t.src0, ping[0] and ping[1] set).  At 512^3 one CTA alone took 23
+// us, the two kernels take 9.
+template <int DT, bool BR>
+cudaError_t launch_staged_tail(TailArgs t, cudaStream_t s) {
+  const uint64_t texels = level_texels(t.n, t.m_top);
+  if (texels > kTailSourceTexels) {
+    const int k = std::min(kGroupLevels, t.levels - 1 - t.m_top);
+    mip_staged_group_kernel<DT, BR><<<(unsigned)(texels >> (3 * k)), 256, 0, s>>>(t, k);
+    const cudaError_t e = cudaGetLastError();
+    t.m_top += k;
+    if (e != cudaSuccess || t.m_top >= t.levels - 1) return e;
+    t.src0 = t.ping[0];
+    std::swap(t.ping[0], t.ping[1]);
+  }
+  mip_tail_kernel<DT, BR><<<1, 1024, 0, s>>>(t);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_build_aniso(const float *level0, const vct_pyramid &pyr, int sms,
@@ -1125,7 +1179,7 @@ cudaError_t launch_build_aniso(const float *level0, const vct_pyramid &pyr, int 
   return e;
 }
 
-// Dense pyramids from a 32-byte aligned grid, n >= 32 (binary16: n <= 256):
+// Dense pyramids from a 32-byte aligned grid, n >= 32:
 // stream_levels_kernel (levels 0 .. 4), then, for float32, groups of
 // kGroupLevels levels while the level below holds more than one tail CTA's
 // worth of texels, then the one-CTA tail (binary16: from the float32 copy of
@@ -1207,13 +1261,13 @@ static cudaError_t build_dense_streamed(const float *level0, const vct_pyramid &
   // levels above m+1 are at most 1/8 of staging_off[1] and land at the start
   // of staging_off[0], whose values were consumed
   t.ping[1] = reinterpret_cast<float4 *>(base + L.staging_off[0]);
+  if (level_texels(pyr.n, m) > kTailSourceTexels) return launch_staged_tail<VCT_F16, false>(t, s);
   return cudaLaunchKernelEx(&lc, mip_tail_kernel<VCT_F16, false, true>, t);
 }
 
 bool streamed_build(const float *level0, const vct_pyramid &pyr) {
   // (its 32-byte loads need a 32-byte aligned grid; the TMA path needs 16)
   return pyr.layout == VCT_LAYOUT_DENSE && pyr.n >= 32 &&
-         (pyr.dtype == VCT_F32 || (pyr.dtype == VCT_F16 && pyr.n <= 256)) &&
          reinterpret_cast<uintptr_t>(level0) % 32 == 0;
 }
 
@@ -1290,12 +1344,8 @@ cudaError_t launch_pack_mips(const float *level0, const vct_pyramid &pyr,
     // Levels above m_top+1 are at most 1/8 of the staging_off[1] region and
     // land at the start of staging_off[0], whose values were consumed.
     t.ping[1] = reinterpret_cast<float4 *>(base + L.staging_off[0]);
-    if (pyr.dtype == VCT_F32)
-      mip_tail_kernel<VCT_F32, true><<<1, 1024, 0, s>>>(t);
-    else if (br)
-      mip_tail_kernel<VCT_F16, true><<<1, 1024, 0, s>>>(t);
-    else
-      mip_tail_kernel<VCT_F16, false><<<1, 1024, 0, s>>>(t);
+    if (pyr.dtype == VCT_F32) return launch_staged_tail<VCT_F32, true>(t, s);
+    return br ? launch_staged_tail<VCT_F16, true>(t, s) : launch_staged_tail<VCT_F16, false>(t, s);
   }
   return cudaGetLastError();
 }

@@ -147,3 +147,19 @@ def test_forward_shapes(w, h, spec, occ, nd, rough, dtype, layout, flags):
     for x, y in ((a.out_diffuse, b.out_diffuse), (a.out_radiance, b.out_radiance)):
         if x is not None:
             assert (x - y).abs().max() <= 32 * 2.0 ** -24 * max(1.0, float(y.abs().max()))
+
+
+# Sizes whose level 4 passes one tail CTA's 4096 texels, whole and cut off
+# inside the levels that several CTAs make: the streaming build and the
+# block-wise one (a grid 16 bytes past a 32-byte boundary) give the same bits.
+@pytest.mark.parametrize("levels", [5, 6, 7, 9, 10])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_large_build_paths_agree(levels, dtype):
+    n = 512
+    buf = torch.empty(4 * n ** 3 + 8, device="cuda")
+    buf[4:4 + 4 * n ** 3].uniform_(generator=torch.Generator(device="cuda").manual_seed(5))
+    shifted = buf[4:4 + 4 * n ** 3].view(n, n, n, 4)
+    a = vct.build_mips(shifted, levels=levels, dtype=dtype)
+    b = vct.build_mips(shifted.clone(), levels=levels, dtype=dtype)
+    for l in range(levels):
+        assert torch.equal(vct.read_level(a, l), vct.read_level(b, l)), l
