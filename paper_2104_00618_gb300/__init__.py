@@ -292,7 +292,8 @@ class View:
 
 
 def _workspace(nbytes: int, device) -> torch.Tensor:
-    return torch.zeros(max(256, nbytes), dtype=torch.uint8, device=device)
+    # (vct_trace clears the counters itself)
+    return torch.empty(max(256, nbytes), dtype=torch.uint8, device=device)
 
 
 def read_stats(workspace: torch.Tensor) -> dict:

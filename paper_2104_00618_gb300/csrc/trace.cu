@@ -559,32 +559,34 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
 inline size_t step_table_bytes(int n_pyr) { return (size_t)n_pyr * 2 * kStepTab * sizeof(float4); }
 
 template <int LPP, int DT, bool BR, bool AN = false>
-cudaError_t launch_t(const TraceLaunch &L, int grid, cudaStream_t s) {
+cudaError_t launch_t(const TraceLaunch &L, int grid, int threads, cudaStream_t s) {
   const size_t dyn = step_table_bytes(L.n_pyr);
   if constexpr (LPP == 1) {
     if (L.group) {
       if (L.var.flags)
-        trace_split_kernel<DT, true, BR, AN><<<grid, kSplitThreads, dyn, s>>>(L);
+        trace_split_kernel<DT, true, BR, AN><<<grid, threads, dyn, s>>>(L);
       else
-        trace_split_kernel<DT, false, BR, AN><<<grid, kSplitThreads, dyn, s>>>(L);
+        trace_split_kernel<DT, false, BR, AN><<<grid, threads, dyn, s>>>(L);
       return cudaGetLastError();
     }
   }
   if (L.var.flags)
-    trace_kernel<LPP, DT, true, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
+    trace_kernel<LPP, DT, true, BR, AN><<<grid, threads, dyn, s>>>(L);
   else
-    trace_kernel<LPP, DT, false, BR, AN><<<grid, kFwdThreads, dyn, s>>>(L);
+    trace_kernel<LPP, DT, false, BR, AN><<<grid, threads, dyn, s>>>(L);
   return cudaGetLastError();
 }
 
 // Anisotropic pyramids are float32 and dense (no brick instance).
 template <int LPP, int DT>
-cudaError_t launch_l(const TraceLaunch &L, bool br, int grid, cudaStream_t s, bool an) {
+cudaError_t launch_l(const TraceLaunch &L, bool br, int grid, int threads, cudaStream_t s,
+                     bool an) {
   if constexpr (DT == VCT_F32) {
-    if (an) return launch_t<LPP, DT, false, true>(L, grid, s);
+    if (an) return launch_t<LPP, DT, false, true>(L, grid, threads, s);
   }
   if (an) return cudaErrorInvalidValue;
-  return br ? launch_t<LPP, DT, true>(L, grid, s) : launch_t<LPP, DT, false>(L, grid, s);
+  return br ? launch_t<LPP, DT, true>(L, grid, threads, s)
+            : launch_t<LPP, DT, false>(L, grid, threads, s);
 }
 
 template <int LPP, int DT>
@@ -604,15 +606,14 @@ int occ_t(bool var) {
 static_assert(sizeof(TraceLaunch) <= 32000, "trace launch parameters exceed the 32 KB limit");
 
 cudaError_t launch_trace(const TraceLaunch &L, int lpp, int dtype, bool bricks, int grid,
-                         cudaStream_t s, bool aniso) {
-  const bool h = dtype == VCT_F16;
-  const bool b = bricks;
-  const bool a = aniso;
+                         int threads, cudaStream_t s, bool aniso) {
+  const bool h = dtype == VCT_F16, b = bricks, a = aniso;
+  const int t = threads;
   switch (lpp) {
-    case 1: return h ? launch_l<1, VCT_F16>(L, b, grid, s, a) : launch_l<1, VCT_F32>(L, b, grid, s, a);
-    case 2: return h ? launch_l<2, VCT_F16>(L, b, grid, s, a) : launch_l<2, VCT_F32>(L, b, grid, s, a);
-    case 4: return h ? launch_l<4, VCT_F16>(L, b, grid, s, a) : launch_l<4, VCT_F32>(L, b, grid, s, a);
-    case 8: return h ? launch_l<8, VCT_F16>(L, b, grid, s, a) : launch_l<8, VCT_F32>(L, b, grid, s, a);
+    case 1: return h ? launch_l<1, VCT_F16>(L, b, grid, t, s, a) : launch_l<1, VCT_F32>(L, b, grid, t, s, a);
+    case 2: return h ? launch_l<2, VCT_F16>(L, b, grid, t, s, a) : launch_l<2, VCT_F32>(L, b, grid, t, s, a);
+    case 4: return h ? launch_l<4, VCT_F16>(L, b, grid, t, s, a) : launch_l<4, VCT_F32>(L, b, grid, t, s, a);
+    case 8: return h ? launch_l<8, VCT_F16>(L, b, grid, t, s, a) : launch_l<8, VCT_F32>(L, b, grid, t, s, a);
     default: return cudaErrorInvalidValue;
   }
 }

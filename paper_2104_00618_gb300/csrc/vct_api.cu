@@ -352,18 +352,19 @@ int64_t total_pixels(const vct_view *views, int32_t n_views) {
 // Tile of a launch that the caller gives no shape for.  Where the specular
 // aperture follows the roughness, a larger tile sorts more cones by length;
 // a smaller one leaves less idle in the last wave of warps.  Measured (9 + 1
-// + 1 cones, 256^3), 8 x 8 / 8 x 16 / 16 x 16: 0.41 M pixels 1671 / 1598 / 2049
-// us, 0.92 M 3307 / 3175 / 3631, 2.07 M 7153 / 6649 / 6880, 3.69 M 12467 /
-// 11544 / 11082 (binary16, bricks, shaded and anisotropic alike within a
-// tenth of that line); one aperture (6 + 1 cones, 64^3): 0.52 M 656 / 704 /
-// 804, 2.07 M 2373 / 2398 / 2596.
+// + 1 cones, 256^3), 8 x 8 / 8 x 16 / 8 x 24 / 16 x 16: 0.41 M pixels 1671 /
+// 1598 / - / 2049 us, 0.92 M 3189 / 2994 / 3088 / 3131, 1.44 M (means of eight
+// scenes) 4583 / 4286 / 4238 / 4467, 2.07 M 6480 / 6015 / 5980 / 6141 (binary16
+// 7034 / 6517 / 6461 / 6644), 3.69 M 12467 / 11544 / - / 11082; one aperture
+// (6 + 1 cones, 64^3): 0.52 M 656 / 704 / - / 804, 2.07 M 2373 / 2398 / - / 2596.
 vct_launch_config default_cfg(const vct_view *views, int32_t n_views, const vct_trace_params &P) {
   bool rough = false;
   for (int i = 0; i < n_views; ++i) rough |= views[i].roughness != nullptr;
   if (!P.spec_enable || !rough || P.spec_aperture_min == P.spec_aperture_max)
     return vct_launch_config{8, 8, 1, 0};
-  if (total_pixels(views, n_views) < 2500000) return vct_launch_config{8, 16, 1, 0};
-  return vct_launch_config{16, 16, 1, 0};
+  const int64_t pixels = total_pixels(views, n_views);
+  if (pixels < 1000000) return vct_launch_config{8, 16, 1, 0};
+  return pixels < 3000000 ? vct_launch_config{8, 24, 1, 0} : vct_launch_config{16, 16, 1, 0};
 }
 
 vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs,
@@ -660,20 +661,28 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
                   "vct_trace: views of one call must use pyramids of one dtype, and all or "
                   "none anisotropic");
     L->n_views = nv;
-    int grid = std::max(1, std::min(cursor, per_sm * sms));
+    int grid = std::max(1, std::min(cursor, per_sm * sms)), threads = kFwdThreads;
     // about two waves of the launch's warps, in small tiles, at the end
     const int64_t tail_px = (int64_t)2 * grid * (kFwdThreads / 32) * kSmallTileW * kSmallTileH;
     if (L->group) {
       L->total_tiles = L->n_big = cursor;
       const int per_cta = kSplitThreads / 32 / L->group;  // tiles a CTA takes at a time
       grid = std::max(1, std::min((cursor + per_cta - 1) / per_cta, kSplitBlocks * sms));
+      threads = kSplitThreads;
     } else {
       L->total_tiles = assign_tail_tiles(L->views, nv, cfg.tile_w, cfg.tile_h, tail_px, L->n_big);
+      // fewer tiles than warps: as few warps per CTA as spreads them over the
+      // SMs (the first CTAs' warps would take them all)
+      const int warps = (L->total_tiles + sms - 1) / sms;
+      if (cfg.ctas_per_sm == 0 && warps < kFwdThreads / 32) {
+        threads = 32 * std::max(1, warps);
+        grid = std::max(1, (L->total_tiles + warps - 1) / std::max(1, warps));
+      }
     }
     if (v0 > 0 && (e = cudaMemsetAsync(L->queue, 0, 4, stream)) != cudaSuccess)
       return cuda_fail(e, "vct_trace queue clear");
     e = launch_trace(*L, cfg.lanes_per_pixel, pyrs[views[v0].pyramid].dtype, bricks, grid,
-                     stream, aniso);
+                     threads, stream, aniso);
     if (e != cudaSuccess) return cuda_fail(e, "vct_trace launch");
   }
   return VCT_OK;

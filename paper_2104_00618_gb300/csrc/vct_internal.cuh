@@ -426,8 +426,9 @@ cudaError_t launch_mip_adjoint_aniso(const vct_pyramid &pyr, const float *gpyr_b
 cudaError_t launch_wait_probe(uint32_t *flag, uint64_t max_ns, cudaStream_t s);
 cudaError_t launch_bounds_probe(uint32_t *buf, uint32_t declared, uint32_t extra,
                                 cudaStream_t s);
+// `threads`: of a CTA, at most kFwdThreads (kSplitThreads where L.group is set).
 cudaError_t launch_trace(const TraceLaunch &L, int lpp, int dtype, bool bricks, int grid,
-                         cudaStream_t s, bool aniso = false);
+                         int threads, cudaStream_t s, bool aniso = false);
 int trace_occupancy(int lpp, int dtype, bool variants);
 cudaError_t launch_trace_bwd(const BwdLaunch &L, int lpp, int grid, cudaStream_t s);
 // Fixed-point gradient (units of 2^-32) -> float32, `count` values.
