@@ -558,6 +558,18 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
 // Dynamic shared memory of a launch: the step tables of its pyramids.
 inline size_t step_table_bytes(int n_pyr) { return (size_t)n_pyr * 2 * kStepTab * sizeof(float4); }
 
+// Static shared memory of trace_kernel.  With the tables of five pyramids and
+// more a CTA passes the 48 KB of a plain launch; the limit asked for is always
+// that of VCT_MAX_PYRAMIDS, so that callers on other threads do not lower it.
+constexpr size_t kTraceStatic = kSpreadLut * sizeof(uint2) + kFwdThreads / 32 * kMaxSortPixels * 4;
+
+template <typename K>
+cudaError_t allow_shared(K kernel, size_t dyn) {
+  if (kTraceStatic + dyn <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(step_table_bytes(VCT_MAX_PYRAMIDS)));
+}
+
 template <int LPP, int DT, bool BR, bool AN = false>
 cudaError_t launch_t(const TraceLaunch &L, int grid, int threads, cudaStream_t s) {
   const size_t dyn = step_table_bytes(L.n_pyr);
@@ -570,10 +582,13 @@ cudaError_t launch_t(const TraceLaunch &L, int grid, int threads, cudaStream_t s
       return cudaGetLastError();
     }
   }
-  if (L.var.flags)
+  if (L.var.flags) {
+    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, true, BR, AN>, dyn)) return e;
     trace_kernel<LPP, DT, true, BR, AN><<<grid, threads, dyn, s>>>(L);
-  else
+  } else {
+    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, false, BR, AN>, dyn)) return e;
     trace_kernel<LPP, DT, false, BR, AN><<<grid, threads, dyn, s>>>(L);
+  }
   return cudaGetLastError();
 }
 

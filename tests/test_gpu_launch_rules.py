@@ -149,6 +149,42 @@ def test_forward_shapes(w, h, spec, occ, nd, rough, dtype, layout, flags):
             assert (x - y).abs().max() <= 32 * 2.0 ** -24 * max(1.0, float(y.abs().max()))
 
 
+# Four, five and all eight pyramids of a call: from five up the step tables
+# pass the shared memory of a plain launch.  Each view alone gives the same
+# bits.
+@pytest.mark.parametrize("n_pyr", [4, 5, 8])
+@pytest.mark.parametrize("lpp,cfg", [(1, True), (1, False), (4, True)])
+@pytest.mark.parametrize("layout,flags", [("dense", 0), ("bricks", 0), ("aniso", 0), ("dense", 15)])
+def test_many_pyramids(n_pyr, lpp, cfg, layout, flags):
+    rng = np.random.default_rng(n_pyr)
+    scene = vs.box_scene(16, 4, 5, room=True)
+    view = vs.interior_view(scene, 40, 37, rng, with_roughness=True)
+    dirs, wts = vs.cone_table_ring6()
+    prm = vs.trace_params(dirs, wts, 1.0, spec_enable=1, spec_aperture_min=0.3,
+                          spec_aperture_max=0.9, occ_enable=1, light=scene["light"])
+    prm = vs.variant_params(prm, flags)
+    grid = torch.from_numpy(scene["grid"]).cuda()
+    P = [vct.build_mips(grid * (0.5 + 0.05 * i), layout=layout) for i in range(n_pyr)]
+    shape = vct.launch_config(8, 8, lpp) if cfg else None
+
+    def make(i):
+        v = vct.View.from_host({**view, "pyramid": i})
+        if flags:
+            v.albedo = torch.full((40 * 37, 3), 0.7, device="cuda")
+            v.alloc_outputs(radiance=True)
+        return v
+
+    got = [make(i) for i in range(n_pyr)]
+    vct.trace(P, got, prm, cfg=shape)
+    for i in range(n_pyr):
+        one = make(0)
+        vct.trace([P[i]], [one], prm, cfg=shape or vct.launch_config(8, 8, 1))
+        assert torch.equal(got[i].out_specular, one.out_specular)
+        assert torch.equal(got[i].out_visibility, one.out_visibility)
+        d = (got[i].out_diffuse - one.out_diffuse).abs().max()
+        assert d <= (0 if cfg else 32 * 2.0 ** -24 * max(1.0, float(one.out_diffuse.abs().max())))
+
+
 # Sizes whose level 4 passes one tail CTA's 4096 texels, whole and cut off
 # inside the levels that several CTAs make: the streaming build and the
 # block-wise one (a grid 16 bytes past a 32-byte boundary) give the same bits.
