@@ -194,9 +194,10 @@ __global__ void __launch_bounds__(kFwdThreads, kTraceMinBlocks) trace_kernel(con
   const int first_cone = defer_spec ? 1 : 0;  // the specular cone is cone 0
   const float T0 = L.spec.t0_vox;
   __shared__ uint2 s_lut[kSpreadLut];
-  __shared__ uint32_t s_keys[kFwdThreads / 32][kMaxSortPixels];
-  extern __shared__ __align__(16) float4 s_tab[];  // n_pyr * 2 * kStepTab entries
-  uint32_t *keys = s_keys[threadIdx.x >> 5];
+  // n_pyr * 2 * kStepTab entries, then kMaxSortPixels keys per warp
+  extern __shared__ __align__(16) float4 s_tab[];
+  uint32_t *keys = reinterpret_cast<uint32_t *>(s_tab + L.n_pyr * 2 * kStepTab) +
+                   (threadIdx.x >> 5) * kMaxSortPixels;
   fill_step_table(s_tab, L.pyr, L.n_pyr, T0);
   fill_spread_lut(s_lut);  // (its barrier also covers s_tab)
 
@@ -558,16 +559,19 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
 // Dynamic shared memory of a launch: the step tables of its pyramids.
 inline size_t step_table_bytes(int n_pyr) { return (size_t)n_pyr * 2 * kStepTab * sizeof(float4); }
 
+// and the sort keys of its warps, behind them (trace_kernel).
+inline size_t sort_key_bytes(int threads) { return (size_t)threads / 32 * kMaxSortPixels * 4; }
+
 // Static shared memory of trace_kernel.  With the tables of five pyramids and
 // more a CTA passes the 48 KB of a plain launch; the limit asked for is always
 // that of VCT_MAX_PYRAMIDS, so that callers on other threads do not lower it.
-constexpr size_t kTraceStatic = kSpreadLut * sizeof(uint2) + kFwdThreads / 32 * kMaxSortPixels * 4;
+constexpr size_t kTraceStatic = kSpreadLut * sizeof(uint2);
 
 template <typename K>
 cudaError_t allow_shared(K kernel, size_t dyn) {
   if (kTraceStatic + dyn <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(step_table_bytes(VCT_MAX_PYRAMIDS)));
+                              (int)(step_table_bytes(VCT_MAX_PYRAMIDS) + sort_key_bytes(kFwdThreads)));
 }
 
 template <int LPP, int DT, bool BR, bool AN = false>
@@ -582,12 +586,13 @@ cudaError_t launch_t(const TraceLaunch &L, int grid, int threads, cudaStream_t s
       return cudaGetLastError();
     }
   }
+  const size_t all = dyn + sort_key_bytes(threads);
   if (L.var.flags) {
-    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, true, BR, AN>, dyn)) return e;
-    trace_kernel<LPP, DT, true, BR, AN><<<grid, threads, dyn, s>>>(L);
+    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, true, BR, AN>, all)) return e;
+    trace_kernel<LPP, DT, true, BR, AN><<<grid, threads, all, s>>>(L);
   } else {
-    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, false, BR, AN>, dyn)) return e;
-    trace_kernel<LPP, DT, false, BR, AN><<<grid, threads, dyn, s>>>(L);
+    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, false, BR, AN>, all)) return e;
+    trace_kernel<LPP, DT, false, BR, AN><<<grid, threads, all, s>>>(L);
   }
   return cudaGetLastError();
 }
@@ -609,10 +614,14 @@ int occ_t(bool var) {
   int b = 0;
   if (var)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, trace_kernel<LPP, DT, true, false, false>,
-                                                  kFwdThreads, step_table_bytes(VCT_MAX_PYRAMIDS));
+                                                  kFwdThreads,
+                                                  step_table_bytes(VCT_MAX_PYRAMIDS) +
+                                                      sort_key_bytes(kFwdThreads));
   else
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, trace_kernel<LPP, DT, false, false, false>,
-                                                  kFwdThreads, step_table_bytes(VCT_MAX_PYRAMIDS));
+                                                  kFwdThreads,
+                                                  step_table_bytes(VCT_MAX_PYRAMIDS) +
+                                                      sort_key_bytes(kFwdThreads));
   return b;
 }
 

@@ -355,16 +355,25 @@ int64_t total_pixels(const vct_view *views, int32_t n_views) {
 // + 1 cones, 256^3), 8 x 8 / 8 x 16 / 8 x 24 / 16 x 16: 0.41 M pixels 1671 /
 // 1598 / - / 2049 us, 0.92 M 3189 / 2994 / 3088 / 3131, 1.44 M (means of eight
 // scenes) 4583 / 4286 / 4238 / 4467, 2.07 M 6480 / 6015 / 5980 / 6141 (binary16
-// 7034 / 6517 / 6461 / 6644), 3.69 M 12467 / 11544 / - / 11082; one aperture
+// 7034 / 6517 / 6461 / 6644), 3.69 M 12467 / 11544 / - / 11082 (all with one
+// CTA per SM; with two, as dense float32 takes for the last two tiles, 1.44 M
+// 4315 / 4365 / 4371 without the first, 2.07 M 6082 / 6017 / 6068); one aperture
 // (6 + 1 cones, 64^3): 0.52 M 656 / 704 / - / 804, 2.07 M 2373 / 2398 / - / 2596.
-vct_launch_config default_cfg(const vct_view *views, int32_t n_views, const vct_trace_params &P) {
+vct_launch_config default_cfg(const vct_pyramid *pyrs, const vct_view *views, int32_t n_views,
+                              const vct_trace_params &P) {
   bool rough = false;
   for (int i = 0; i < n_views; ++i) rough |= views[i].roughness != nullptr;
   if (!P.spec_enable || !rough || P.spec_aperture_min == P.spec_aperture_max)
     return vct_launch_config{8, 8, 1, 0};
   const int64_t pixels = total_pixels(views, n_views);
   if (pixels < 1000000) return vct_launch_config{8, 16, 1, 0};
-  return pixels < 3000000 ? vct_launch_config{8, 24, 1, 0} : vct_launch_config{16, 16, 1, 0};
+  // (dense float32 at 1.44 M, two CTAs: 8 x 24 5.40 ms, 16 x 16 5.30 in a room
+  // of surface shells, 4365 and 4371 us as above; at 2.07 M 7.37 - 7.49 and
+  // 7.36 - 7.57 ms, 6017 and 6068 us)
+  const vct_pyramid &p0 = pyrs[views[0].pyramid];
+  const int64_t lower = p0.dtype == VCT_F32 && p0.layout == VCT_LAYOUT_DENSE && !P.flags ? 1750000 : 0;
+  return pixels >= lower && pixels < 3000000 ? vct_launch_config{8, 24, 1, 0}
+                                             : vct_launch_config{16, 16, 1, 0};
 }
 
 vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs,
@@ -375,7 +384,7 @@ vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs
   std::lock_guard<std::mutex> g(g_tune_mu);
   auto it = g_tuned.find(tune_key(pyrs, views, P));
   tuned = it != g_tuned.end();
-  return tuned ? it->second : default_cfg(views, n_views, *P);
+  return tuned ? it->second : default_cfg(pyrs, views, n_views, *P);
 }
 
 // Warps that share a tile's cones in a launch whose shape is the library's
@@ -677,6 +686,17 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
       if (cfg.ctas_per_sm == 0 && warps < kFwdThreads / 32) {
         threads = 32 * std::max(1, warps);
         grid = std::max(1, (L->total_tiles + warps - 1) / std::max(1, warps));
+      }
+      // Large tiles of dense float32 frames: as many warps in two CTAs of half
+      // the size.  1080p, one / two CTAs per SM, 8 x 24 tiles: six views of
+      // meshes' surface shells 6.59 - 7.64 / 6.48 - 7.49 ms, filled boxes (mean
+      // of eight) 5.98 / 6.02; 16 x 16: 6.73 - 7.84 / 6.45 - 7.57, 6.14 / 6.07.
+      // Small tiles and the other kernels take one: 8 x 16 7.49 / 7.59,
+      // binary16 6.49 / 6.57, anisotropic (128^3) 2.87 / 3.03, shaded 3.47 / 3.53.
+      if (cfg.ctas_per_sm == 0 && threads == kFwdThreads && cfg.tile_w * cfg.tile_h >= 192 &&
+          pyrs[views[v0].pyramid].dtype == VCT_F32 && !bricks && !aniso && !params->flags) {
+        threads = kFwdThreads / 2;
+        grid = std::max(1, std::min(2 * grid, (L->total_tiles + threads / 32 - 1) / (threads / 32)));
       }
     }
     if (v0 > 0 && (e = cudaMemsetAsync(L->queue, 0, 4, stream)) != cudaSuccess)

@@ -15,8 +15,9 @@ constexpr int kTraceThreads = 256;      // CTA shape of the adjoint trace kernel
 // Forward trace CTAs: warps work independently, so the CTA size sets the
 // register budget, 65536 / (kFwdThreads * kTraceMinBlocks) per thread, and the
 // copies of the Morton tables per SM: one CTA of 512 threads leaves 24 KB more
-// to the L1 than two of 256 (1080p frame 5.83 -> 5.57 ms, binary16 128^3 2.51
-// -> 2.39, anisotropic 3.04 -> 2.88).
+// to the L1 than two of 256 (binary16 128^3 frame 2.51 -> 2.37 ms, anisotropic
+// 3.03 -> 2.87).  Large tiles of dense float32 frames take two all the same
+// (vct_trace's launch has the figures).
 #ifndef VCT_FWD_THREADS
 #define VCT_FWD_THREADS 512
 #endif

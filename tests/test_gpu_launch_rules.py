@@ -149,6 +149,33 @@ def test_forward_shapes(w, h, spec, occ, nd, rough, dtype, layout, flags):
             assert (x - y).abs().max() <= 32 * 2.0 ** -24 * max(1.0, float(y.abs().max()))
 
 
+# Tiles of 192 pixels and more of dense float32 frames run in two CTAs of half
+# the size per SM, just below that in one; an explicit CTA count keeps one.
+# The same pixels in the same warps' order: the same bits.  Eight pyramids
+# take the most shared memory.
+@pytest.mark.parametrize("tile,views", [((8, 24), 1), ((16, 16), 1), ((8, 23), 1), ((12, 16), 8)])
+def test_forward_cta_sizes(tile, views):
+    w, h = 1001, 701
+    rng = np.random.default_rng(views)
+    scene = vs.box_scene(16, 4, 5, room=True)
+    dirs, wts = vs.cone_table_ring6()
+    prm = vs.trace_params(dirs[:2], wts[:2], 1.0, spec_enable=1, spec_aperture_min=0.3,
+                          spec_aperture_max=0.9, occ_enable=1, light=scene["light"])
+    P = [vct.build_mips(torch.from_numpy(scene["grid"]).cuda()) for _ in range(views)]
+    host = vs.interior_view(scene, w, h, rng, with_roughness=True)
+    out = []
+    for per_sm in (0, 1):
+        v = [vct.View.from_host({**host, "pyramid": i}) for i in range(views)]
+        stats = vct.read_stats(vct.trace(P, v, prm, cfg=vct.launch_config(*tile, 1, per_sm)))
+        out.append((v, stats))
+    (a, sa), (b, sb) = out
+    assert sa == sb
+    for x, y in zip(a, b):
+        assert torch.equal(x.out_diffuse, y.out_diffuse)
+        assert torch.equal(x.out_specular, y.out_specular)
+        assert torch.equal(x.out_visibility, y.out_visibility)
+
+
 # Four, five and all eight pyramids of a call: from five up the step tables
 # pass the shared memory of a plain launch.  Each view alone gives the same
 # bits.
