@@ -510,9 +510,9 @@ def extra_small(torch, vct, dev):
     for dt in ("f32", "f16"):
         P = vct.Pyramid(scene["n"], None, dt, device=dev)
         vct.build_mips(level0, out=P)
-        # 16 K pixels fill few of the default 16x16 tiles: let the library's
-        # tuner pick the tile and lanes per pixel for this shape (vct_trace
-        # then uses its choice)
+        # the library's tuner: vct_trace then uses the fastest shape, or keeps
+        # its own rules by size where no candidate beats them ("tuned" is the
+        # fastest candidate either way)
         tuned = vct.autotune([P], [view], params, workspace=ws)
         tr_ms = _time(torch, lambda: vct.trace([P], [view], params, workspace=ws), 50, warm=5)
         st_ms = _time(torch, lambda: (vct.build_mips(level0, out=P),

@@ -377,12 +377,17 @@ vct_status vct_trace(const vct_pyramid *pyrs, int32_t n_pyramids,
                      size_t workspace_bytes, vct_stream_t stream);
 
 /*
- * Times every candidate launch shape (tile 4x8, 8x8, 8x16, 16x16 x
- * lanes_per_pixel 1, 2, 4, 8) on the given views, synchronously, and caches
- * the fastest under (device, dtype of pyrs[0], n of pyrs[0], tracing of the
- * specular/occlusion cones); vct_trace with cfg == NULL then uses it.  The
- * views' outputs are overwritten.  `best` (host, may be NULL) receives the
- * choice.
+ * Times the shape vct_trace picks by itself for the given views and every
+ * candidate shape (tile 4x8, 8x8, 8x16, 8x24, 16x16 x lanes_per_pixel 1, 2, 4,
+ * 8), synchronously.  If a candidate is more than 3 % faster than the
+ * library's own pick, vct_trace with cfg == NULL uses it from then on under
+ * the same key: device, dtype, layout and n of pyrs[0], numbers of diffuse,
+ * specular and occlusion cones, presence of roughness in views[0], whether
+ * the specular aperture varies, flags, and whether the call has so few pixels
+ * that warps share tiles (and how many do).  Otherwise the key goes back to
+ * the library's pick, which follows each call's size.  The views' outputs are
+ * overwritten.  `best` (host, may be NULL) receives the fastest candidate
+ * either way.
  */
 vct_status vct_autotune_trace(const vct_pyramid *pyrs, int32_t n_pyramids,
                               const vct_view *views, int32_t n_views,

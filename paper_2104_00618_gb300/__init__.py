@@ -320,6 +320,9 @@ def trace(pyramids, views, params, cfg: VctLaunchConfig | None = None,
 
 
 def autotune(pyramids, views, params, workspace=None, stream=None) -> VctLaunchConfig:
+    """Times the launch shapes on these views (outputs are overwritten) and
+    returns the fastest one with a tile of its own; later trace() calls of this
+    kind without a shape use it if it beats the library's pick (vct.h)."""
     pyrs = list(pyramids) if isinstance(pyramids, (list, tuple)) else [pyramids]
     vs = list(views) if isinstance(views, (list, tuple)) else [views]
     P = params if isinstance(params, VctTraceParams) else make_params(params)

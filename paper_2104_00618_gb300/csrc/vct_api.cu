@@ -4,6 +4,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -12,7 +13,6 @@
 #include <memory>
 #include <mutex>
 #include <string>
-#include <tuple>
 #include <vector>
 
 #include "gbuffer.cuh"
@@ -331,16 +331,45 @@ bool cfg_ok(const vct_launch_config &c) {
          c.ctas_per_sm <= 32;
 }
 
-// Launch-shape cache filled by vct_autotune_trace.
-using TuneKey = std::tuple<int, int, int, int, int, int, int>;
+// Warps that share a tile's cones in a launch whose shape is the library's
+// choice, or 0 (each warp takes whole tiles).  A warp that marches all cones
+// of its 32 pixels in series takes the same time however few pixels there
+// are, so the cones of a launch of few warps are split: four ways while its
+// warps are then no more than the chip holds at once, two ways up to four
+// times that.  Measured, split 4 / 2 / 1 ways: 9 + 1 + 1 cones at 256^3, 5917
+// pixels 141 / 210 / 318 us, 16 384: 173 / 204 / 304, 25 600: 240 / 252 / 299,
+// 57 600: 396 / 399 / 407, 129 600: 758 / 689 / 695, 230 400 (the last in 8 x
+// 16 tiles): 1271 / 1135 / 1032; 6 + 1 cones at 64^3, 16 384: 73 / 75 / 107,
+// 57 600: 142 / 121 / 144, 129 600: 269 / 210 / 229.
+int trace_group(const vct_view *views, int32_t n_views, const vct_trace_params &P, int sms) {
+  const int others = P.n_diffuse + P.occ_enable;
+  if (others + P.spec_enable < 2) return 0;
+  int64_t tiles = 0;
+  for (int i = 0; i < n_views; ++i)
+    tiles += (int64_t)((views[i].width + kSmallTileW - 1) / kSmallTileW) *
+             ((views[i].height + kSmallTileH - 1) / kSmallTileH);
+  const int64_t warps = (int64_t)sms * kSplitBlocks * (kSplitThreads / 32);
+  if (tiles * 4 <= warps && others >= 3) return 4;
+  return tiles * 2 <= warps * 4 ? 2 : 0;
+}
+
+// Launch-shape cache filled by vct_autotune_trace, for calls where a shape
+// beat the library's own choice.  The key holds what the shape depends on but
+// for the pixel count, so that a probe of a few views tunes a large batch;
+// of that it holds how many warps share a tile (trace_group), so that a shape
+// tuned on many pixels does not keep a small call from sharing its tiles.
+using TuneKey = std::array<int, 11>;
 std::mutex g_tune_mu;
 std::map<TuneKey, vct_launch_config> g_tuned;
 
-TuneKey tune_key(const vct_pyramid *pyrs, const vct_view *views, const vct_trace_params *P) {
+TuneKey tune_key(const vct_pyramid *pyrs, const vct_view *views, int32_t n_views,
+                 const vct_trace_params *P) {
   int dev = 0;
   cudaGetDevice(&dev);
-  return TuneKey(dev, pyrs[0].dtype, pyrs[0].n, P->spec_enable, P->occ_enable,
-                 views[0].roughness != nullptr, P->flags);
+  return TuneKey{dev, pyrs[0].dtype, pyrs[0].layout, pyrs[0].n, P->n_diffuse, P->spec_enable,
+                 P->occ_enable, views[0].roughness != nullptr,
+                 P->spec_aperture_min != P->spec_aperture_max, P->flags,
+                 trace_group(views, n_views, *P, sm_count())};
 }
 
 int64_t total_pixels(const vct_view *views, int32_t n_views) {
@@ -382,31 +411,9 @@ vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs
   tuned = false;
   if (cfg) return *cfg;
   std::lock_guard<std::mutex> g(g_tune_mu);
-  auto it = g_tuned.find(tune_key(pyrs, views, P));
+  auto it = g_tuned.find(tune_key(pyrs, views, n_views, P));
   tuned = it != g_tuned.end();
   return tuned ? it->second : default_cfg(pyrs, views, n_views, *P);
-}
-
-// Warps that share a tile's cones in a launch whose shape is the library's
-// choice, or 0 (each warp takes whole tiles).  A warp that marches all cones
-// of its 32 pixels in series takes the same time however few pixels there
-// are, so the cones of a launch of few warps are split: four ways while its
-// warps are then no more than the chip holds at once, two ways up to four
-// times that.  Measured, split 4 / 2 / 1 ways: 9 + 1 + 1 cones at 256^3, 5917
-// pixels 141 / 210 / 318 us, 16 384: 173 / 204 / 304, 25 600: 240 / 252 / 299,
-// 57 600: 396 / 399 / 407, 129 600: 758 / 689 / 695, 230 400 (the last in 8 x
-// 16 tiles): 1271 / 1135 / 1032; 6 + 1 cones at 64^3, 16 384: 73 / 75 / 107,
-// 57 600: 142 / 121 / 144, 129 600: 269 / 210 / 229.
-int trace_group(const vct_view *views, int32_t n_views, const vct_trace_params &P, int sms) {
-  const int others = P.n_diffuse + P.occ_enable;
-  if (others + P.spec_enable < 2) return 0;
-  int64_t tiles = 0;
-  for (int i = 0; i < n_views; ++i)
-    tiles += (int64_t)((views[i].width + kSmallTileW - 1) / kSmallTileW) *
-             ((views[i].height + kSmallTileH - 1) / kSmallTileH);
-  const int64_t warps = (int64_t)sms * kSplitBlocks * (kSplitThreads / 32);
-  if (tiles * 4 <= warps && others >= 3) return 4;
-  return tiles * 2 <= warps * 4 ? 2 : 0;
 }
 
 struct TraceStatsLayout {
@@ -751,43 +758,48 @@ vct_status vct_autotune_trace(const vct_pyramid *pyrs, int32_t n_pyr, const vct_
   cudaEvent_t e0, e1;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return fail(VCT_ERR_CUDA, "vct_autotune_trace: event create failed");
-  const int tiles[4][2] = {{4, 8}, {8, 8}, {8, 16}, {16, 16}};
-  const int lpps[4] = {1, 2, 4, 8};
-  float best_ms = 1e30f;
-  vct_launch_config bc{16, 16, 1, 0};
-  for (auto &t : tiles)
-    for (int lpp : lpps) {
-      vct_launch_config c{t[0], t[1], lpp, 0};
-      float ms_sum = 0.f;
-      for (int rep = 0; rep < 3; ++rep) {
-        cudaEventRecord(e0, s);
-        st = trace_impl(pyrs, n_pyr, views, n_views, params, c, false, workspace, workspace_bytes, s,
-                        true);
-        cudaEventRecord(e1, s);
-        if (st != VCT_OK) break;
-        if (cudaEventSynchronize(e1) != cudaSuccess) {
-          st = fail(VCT_ERR_CUDA, "vct_autotune_trace: kernel failed");
-          break;
-        }
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        if (rep > 0) ms_sum += ms;  // first run warms caches
-      }
-      if (st != VCT_OK) {
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        return st;
-      }
-      if (ms_sum < best_ms) {
-        best_ms = ms_sum;
-        bc = c;
-      }
+  // The mean of two runs after a first one that warms the caches.
+  auto timed = [&](const vct_launch_config &c, bool any_shape, float &ms) -> vct_status {
+    ms = 0.f;
+    for (int rep = 0; rep < 3; ++rep) {
+      cudaEventRecord(e0, s);
+      const vct_status r = trace_impl(pyrs, n_pyr, views, n_views, params, c, any_shape, workspace,
+                                      workspace_bytes, s, true);
+      cudaEventRecord(e1, s);
+      if (r != VCT_OK) return r;
+      if (cudaEventSynchronize(e1) != cudaSuccess)
+        return fail(VCT_ERR_CUDA, "vct_autotune_trace: kernel failed");
+      float t = 0.f;
+      cudaEventElapsedTime(&t, e0, e1);
+      if (rep > 0) ms += 0.5f * t;
     }
+    return VCT_OK;
+  };
+  const int tiles[5][2] = {{4, 8}, {8, 8}, {8, 16}, {8, 24}, {16, 16}};
+  const int lpps[4] = {1, 2, 4, 8};
+  float own_ms = 0.f, best_ms = 1e30f;
+  vct_launch_config bc{16, 16, 1, 0};
+  st = timed(default_cfg(pyrs, views, n_views, *params), true, own_ms);
+  for (int i = 0; st == VCT_OK && i < 20; ++i) {
+    const vct_launch_config c{tiles[i / 4][0], tiles[i / 4][1], lpps[i % 4], 0};
+    float ms = 0.f;
+    st = timed(c, false, ms);
+    if (st == VCT_OK && ms < best_ms) {
+      best_ms = ms;
+      bc = c;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (st != VCT_OK) return st;
   {
     std::lock_guard<std::mutex> g(g_tune_mu);
-    g_tuned[tune_key(pyrs, views, params)] = bc;
+    const TuneKey key = tune_key(pyrs, views, n_views, params);
+    // (two runs of one shape differ by up to 3 %)
+    if (best_ms < 0.97f * own_ms)
+      g_tuned[key] = bc;
+    else
+      g_tuned.erase(key);
   }
   if (best) *best = bc;
   return VCT_OK;

@@ -3,6 +3,8 @@
 A pixel's sums are the same terms in another order on either side, so every
 case is held to the float32 bound of the repository's other comparisons.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -80,7 +82,6 @@ def test_brick_build_lists(n, fill, dtype, planned):
 
 
 def test_planned_build_checks_its_pool_and_scratch():
-    import ctypes
     lib, abi = vct.lib(), vct._abi
     g = torch.rand((64, 64, 64, 4), device="cuda")
     occ, _ = vct.plan_bricks(g)
@@ -226,3 +227,63 @@ def test_large_build_paths_agree(levels, dtype):
     b = vct.build_mips(shifted.clone(), levels=levels, dtype=dtype)
     for l in range(levels):
         assert torch.equal(vct.read_level(a, l), vct.read_level(b, l)), l
+
+
+class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v1
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3),
+                ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p)]
+
+
+def _launch(P, view, prm, cfg=None):
+    """(CTAs, threads per CTA, work-queue cursor afterwards) of a trace's one
+    kernel.  The cursor counts the items and one last pull by every warp (or
+    group of warps), so it tells tiles apart."""
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        vct.trace(P, view, prm, cfg=cfg, workspace=ws)
+    drv = ctypes.CDLL("libcuda.so.1")
+    raw = ctypes.c_void_p(graph.raw_cuda_graph())
+    count = ctypes.c_size_t()
+    assert drv.cuGraphGetNodes(raw, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert drv.cuGraphGetNodes(raw, nodes, ctypes.byref(count)) == 0
+    kernels = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 0:  # a kernel
+            k = _KernelNode()
+            assert drv.cuGraphKernelNodeGetParams(ctypes.c_void_p(node), ctypes.byref(k)) == 0
+            kernels.append(k)
+    assert len(kernels) == 1
+    graph.replay()
+    queue = int(ws[:56].cpu().numpy().view(np.uint32)[12])
+    return kernels[0].grid[0], kernels[0].block[0], queue
+
+
+# Tuning never leaves a call slower than the library's own pick: not the call
+# it was run for (a shape is kept only if it beat that pick), and not a small
+# call of the same kind, whose warps share tiles.
+@pytest.mark.parametrize("rough", [False, True])
+def test_autotune_leaves_small_calls_alone(rough):
+    scene = vs.box_scene(32, 4, 5, room=True)
+    dirs, wts = vs.cone_table_ring6()
+    prm = vs.trace_params(dirs, wts, 1.0, spec_enable=1, spec_aperture_min=0.3,
+                          spec_aperture_max=0.9, occ_enable=1, light=scene["light"])
+    P = vct.build_mips(torch.from_numpy(scene["grid"]).cuda())
+    rng = np.random.default_rng(3)
+    small, mid, large = (vct.View.from_host(vs.interior_view(scene, w, h, rng,
+                                                             with_roughness=rough))
+                         for w, h in ((100, 91), (270, 200), (1024, 768)))
+    own = [_launch(P, v, prm) for v in (small, mid, large)]
+    for v, o in ((small, own[0]), (mid, own[1])):  # warps that share tiles
+        assert o != _launch(P, v, prm, vct.launch_config(8, 8))
+    best = vct.autotune(P, large, prm)
+    assert _launch(P, small, prm) == own[0] and _launch(P, mid, prm) == own[1]
+    assert _launch(P, large, prm) in (own[2], _launch(P, large, prm, best))
+    # one warp marching a tile's cones in series takes about twice as long as
+    # four sharing them, so no candidate wins here
+    vct.autotune(P, small, prm)
+    assert _launch(P, small, prm) == own[0]
