@@ -192,9 +192,13 @@ vct_status vct_build_mips(const float *level0_dense, const vct_pyramid *pyr,
  * vct_pyramid_plan_bricks: `scratch` still holds what that call left there
  * for the same n, levels, dtype and level0_dense, whose contents are
  * unchanged, and the occupancy is taken from it instead of from another pass
- * over the grid.  Same result and errors as vct_build_mips, and
- * VCT_ERR_INVALID_ARG for another layout, VCT_ERR_WORKSPACE for a NULL, too
- * small or misaligned scratch (vct_pyramid_plan_scratch_bytes()).
+ * over the grid.  The scratch is read on `stream`: it must stay valid and
+ * unchanged until the stream has passed this call.  Same result and errors as
+ * vct_build_mips, and VCT_ERR_INVALID_ARG for another layout,
+ * VCT_ERR_WORKSPACE for a NULL, too small or misaligned scratch
+ * (vct_pyramid_plan_scratch_bytes()).  A scratch without a plan of this n and
+ * levels leaves every brick empty, and a damaged one no slot outside the
+ * pool; vct_pyramid_status() reports VCT_ERR_WORKSPACE for both.
  */
 vct_status vct_build_mips_planned(const float *level0_dense, const vct_pyramid *pyr,
                                   const void *scratch, size_t scratch_bytes,
@@ -220,7 +224,8 @@ vct_status vct_pyramid_read_volume(const vct_pyramid *pyr, int32_t level, int32_
  * pyramid header.  Returns VCT_ERR_TIMEOUT if a kernel that wrote this
  * pyramid gave up a bounded wait (the pyramid contents are then undefined),
  * VCT_ERR_WORKSPACE if a brick pyramid's pool was too small for its occupied
- * bricks (see vct_build_mips), VCT_OK otherwise.
+ * bricks (see vct_build_mips) or its plan was not one of this shape
+ * (vct_build_mips_planned), VCT_OK otherwise.
  */
 vct_status vct_pyramid_status(const vct_pyramid *pyr, vct_stream_t stream);
 

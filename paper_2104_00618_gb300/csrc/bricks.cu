@@ -15,6 +15,7 @@ struct TableArgs {
   int nbricked;                   // bricked levels are 0 .. nbricked-1
   uint32_t *status;
   unsigned long long *count;
+  uint32_t *plan;                 // the tables' shape word (plan_word)
   uint64_t capacity;              // pool bricks, the zero brick included
 };
 
@@ -58,7 +59,7 @@ constexpr int kScanThreads = 1024;
 constexpr int kScanRun = 8;    // consecutive flags per thread and pass
 constexpr int kScanCtas = 56;  // sums in header words 4 .. 59
 constexpr int kScanPass = kScanThreads * kScanRun;
-static_assert(16 + 4 * kScanCtas <= kHeaderBytes, "the parts' sums lie in the header");
+static_assert(16 + 4 * kScanCtas <= kHeaderPlanOff, "the parts' sums lie in the header");
 
 struct ScanArgs {
   uint32_t *flags, *sums;  // sums: null where one pass of one CTA holds every flag
@@ -67,6 +68,8 @@ struct ScanArgs {
   uint32_t *status;
   unsigned long long *count;
   uint64_t capacity;
+  uint32_t *plan;  // the tables' shape word (plan_word)
+  uint32_t plan_value;
 };
 
 __device__ __forceinline__ uint32_t load_flags(const ScanArgs &a, uint64_t e, uint64_t end) {
@@ -126,6 +129,7 @@ __global__ void __launch_bounds__(kScanThreads) slots_kernel(const __grid_consta
   const bool fits = 1ull + total <= a.capacity;  // else: leave every brick empty, report it
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *a.count = total;
+    *a.plan = a.plan_value;
     if (!fits) atomicExch(a.status, (uint32_t)VCT_ERR_WORKSPACE);
   }
   const uint64_t begin = blockIdx.x * a.part, end = min(begin + a.part, a.words);
@@ -169,20 +173,44 @@ __global__ void __launch_bounds__(kScanThreads) slots_kernel(const __grid_consta
 
 // Tables and brick count made elsewhere for the same grid shape (`src`: the
 // words at the tables' place there) into this pyramid; slots_kernel's check
-// of the pool.
+// of the pool.  Those words are the caller's: tables of another shape are
+// taken as a pool too small, and a slot above the count, which slots_kernel
+// never hands out, becomes that of an empty brick, so that no slot outside
+// the pool reaches the kernels that store through it; both are reported.
 __global__ void __launch_bounds__(256) adopt_tables_kernel(const __grid_constant__ TableArgs a,
                                                            const uint4 *src, uint4 *dst,
                                                            uint64_t words,
-                                                           const unsigned long long *count) {
-  const unsigned long long total = *count;
-  const bool fits = 1ull + total <= a.capacity;
+                                                           const unsigned long long *count,
+                                                           const uint32_t *plan,
+                                                           uint32_t plan_value) {
+  const bool same = *plan == plan_value;
+  const unsigned long long total = same ? *count : a.capacity;
+  const bool fits = same && total < a.capacity;  // 1 + total bricks
+  bool bad = false;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < words;
-       i += (uint64_t)gridDim.x * blockDim.x)
-    dst[i] = fits ? src[i] : make_uint4(0u, 0u, 0u, 0u);
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (fits) {
+      v = src[i];
+      if (v.x > total || v.y > total || v.z > total || v.w > total) {
+        bad = true;
+        v = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    dst[i] = v;
+  }
+  if (bad) atomicExch(a.status, (uint32_t)VCT_ERR_WORKSPACE);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *a.count = total;
+    *a.plan = plan_value;
     if (!fits) atomicExch(a.status, (uint32_t)VCT_ERR_WORKSPACE);
   }
+}
+
+// Marks tables made for this shape (the places of a pyramid's tables depend on
+// nothing else).
+uint32_t plan_word(int n, int levels) {
+  return 0x56435400u | (uint32_t)ilog2(n) << 4 | (uint32_t)levels;
 }
 
 }  // namespace
@@ -200,6 +228,7 @@ cudaError_t launch_brick_tables(const float *level0, int n, int levels, const La
     }
   a.status = reinterpret_cast<uint32_t *>(base);
   a.count = reinterpret_cast<unsigned long long *>(base + kHeaderCountOff);
+  a.plan = reinterpret_cast<uint32_t *>(base + kHeaderPlanOff);
   a.capacity = capacity;
   if (a.nbricked == 0) {
     cudaError_t e = cudaMemsetAsync(base + kHeaderCountOff, 0, 8, s);
@@ -218,7 +247,8 @@ cudaError_t launch_brick_tables(const float *level0, int n, int levels, const La
     adopt_tables_kernel<<<grid, 256, 0, s>>>(
         a, reinterpret_cast<const uint4 *>(planned + L.level_off[0]),
         reinterpret_cast<uint4 *>(first), words,
-        reinterpret_cast<const unsigned long long *>(planned + kHeaderCountOff));
+        reinterpret_cast<const unsigned long long *>(planned + kHeaderCountOff),
+        reinterpret_cast<const uint32_t *>(planned + kHeaderPlanOff), plan_word(n, levels));
     return cudaGetLastError();
   }
   // A grid whose flags one pass of one CTA holds (n <= 128) needs two launches.
@@ -239,6 +269,8 @@ cudaError_t launch_brick_tables(const float *level0, int n, int levels, const La
   c.status = a.status;
   c.count = a.count;
   c.capacity = capacity;
+  c.plan = a.plan;
+  c.plan_value = plan_word(n, levels);
   const int parts = (int)((c.words + c.part - 1) / c.part);
   c.bricks0 = a.nb[0];
   if (small) {

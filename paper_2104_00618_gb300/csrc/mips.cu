@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) pack_mips_kernel(const __grid_constant__ 
   // others are zero, which the empty bricks say already (512^3 room, a fifth
   // of the blocks occupied: 840 -> 360 us).  Where the pool was too small
   // every slot is 0 and the blocks are all taken.
-  const bool skip = BR && B == 16 && 1ull + *a.count <= a.capacity;
+  const bool skip = BR && B == 16 && *a.count < a.capacity;  // (and the zero brick)
   for (uint64_t run = blockIdx.x; run < a.nblocks; run += (uint64_t)kBlockRun * gridDim.x) {
     const uint64_t left = (a.nblocks - run + gridDim.x - 1) / gridDim.x;
     int nlist = (int)(left < kBlockRun ? left : kBlockRun);

@@ -587,7 +587,8 @@ vct_status vct_pyramid_status(const vct_pyramid *pyr, vct_stream_t stream) {
     return fail(VCT_ERR_TIMEOUT, "a kernel gave up a bounded wait while building this pyramid");
   if (word == (uint32_t)VCT_ERR_WORKSPACE)
     return fail(VCT_ERR_WORKSPACE,
-                "the brick pool of this pyramid was too small for its occupied bricks");
+                "the brick pool of this pyramid was too small for its occupied bricks, or its "
+                "plan was not one of this shape");
   return VCT_OK;
 }
 

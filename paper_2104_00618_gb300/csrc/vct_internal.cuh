@@ -57,6 +57,7 @@ __host__ __device__ inline int pack_block(int n) { return n < 16 ? n : 16; }
 constexpr int kBrickShift = 9;  // 512 texels per brick
 constexpr int kBrickMinEdge = 16;
 constexpr uint64_t kHeaderCountOff = 8;  // uint64 occupied-brick count in the header
+constexpr int kHeaderPlanOff = 240;      // uint32 shape of the slot tables in the header
 
 __host__ __device__ inline bool level_bricked(int n, int l, int layout) {
   return layout == VCT_LAYOUT_BRICKS && (n >> l) >= kBrickMinEdge;
@@ -413,7 +414,9 @@ cudaError_t launch_build_aniso(const float *level0, const vct_pyramid &pyr, int 
 // goes to base + kHeaderCountOff.  More than `capacity` bricks (zero brick
 // included) leaves every slot 0 and writes VCT_ERR_WORKSPACE to the status word.
 // `planned` (may be null): the base of tables made by an earlier call for the
-// same grid; they are copied instead of computed.
+// same grid; they are copied and checked instead of computed (tables of
+// another shape and slots above their count: VCT_ERR_WORKSPACE in the status
+// word).
 cudaError_t launch_brick_tables(const float *level0, int n, int levels, const Layout &L,
                                 uint8_t *base, uint64_t capacity, cudaStream_t s,
                                 const uint8_t *planned = nullptr);

@@ -108,6 +108,45 @@ def test_planned_build_checks_its_pool_and_scratch():
                                       stream) == abi.VCT_ERR_INVALID_ARG
 
 
+# What a planned build makes of a scratch that is not its plan: one of fewer
+# levels, of another edge, never planned, or with slots beyond its count, must
+# neither store outside the pool (the guard after it) nor go unreported.
+@pytest.mark.parametrize("case", ["levels", "edge", "unplanned", "slots"])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_planned_build_refuses_other_plans(case, dtype):
+    lib, abi = vct.lib(), vct._abi
+    dt = vct.DTYPES[dtype]
+    g = torch.rand((64, 64, 64, 4), device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    occ, nbytes = vct.plan_bricks(g, dtype=dtype)
+    sb = lib.vct_pyramid_plan_scratch_bytes(64, 7, dt)
+    scratch = torch.randint(0, 255, (sb,), dtype=torch.uint8, device="cuda")
+    at = ctypes.c_void_p(scratch.data_ptr())
+    if case != "unplanned":
+        other = torch.rand((32, 32, 32, 4), device="cuda") if case == "edge" else g
+        levels = {"levels": 1, "edge": 6, "slots": 7}[case]
+        assert lib.vct_pyramid_plan_bricks(ctypes.c_void_p(other.data_ptr()), len(other), levels,
+                                           dt, at, sb, None, None, stream) == abi.VCT_OK
+    if case == "slots":
+        tables = scratch[256:256 + 4 * 64].view(torch.int32)
+        tables[:3] = torch.tensor([occ + 1, 2 ** 31 - 1, -1], device="cuda")
+    P = vct.Pyramid(64, dtype=dtype, layout="bricks", occupied=occ)
+    P.storage = torch.full((nbytes + 2 ** 20,), 77, dtype=torch.uint8, device="cuda")
+    P.storage[:256] = 0
+    p = P.struct()
+    p.bytes = nbytes
+    assert lib.vct_build_mips_planned(ctypes.c_void_p(g.data_ptr()), ctypes.byref(p), at, sb,
+                                      stream) == abi.VCT_OK
+    with pytest.raises(vct.VctError) as e:
+        vct.pyramid_status(P)
+    assert e.value.status == abi.VCT_ERR_WORKSPACE
+    assert (P.storage[nbytes:] == 77).all()
+    if case != "slots":
+        assert not vct.read_level(P, 0).any()
+        assert torch.allclose(vct.read_level(P, 6), g.mean(dim=(0, 1, 2)),
+                              rtol=1e-5 if dtype == "f32" else 2e-3)
+
+
 # A launch without a shape shares a tile's cones among 4 warps (up to 608
 # tiles of 8 x 4 pixels on 152 SMs), 2 (up to 4864) or none, where the tile
 # depends on the roughness; each against one warp per 8 x 8 tile: the cones
