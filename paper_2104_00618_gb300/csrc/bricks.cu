@@ -110,11 +110,12 @@ __global__ void __launch_bounds__(kScanThreads) slots_kernel(const __grid_consta
   total = __reduce_add_sync(0xffffffffu, total);
   if (a.sums == nullptr) {  // one part of one pass: the coarser flags and the count here
     const uint32_t *child = a.flags;
-    for (uint64_t nb = a.bricks0 >> 3, at = a.bricks0; nb >= 8; at += nb, nb >>= 3) {
+    // (nb: bricks of the next level, whose flags start at `at`)
+    for (uint64_t nb = a.bricks0 >> 3, at = a.bricks0; at < a.words; at += nb, nb >>= 3) {
       for (uint64_t p = threadIdx.x; p < nb; p += blockDim.x) {
         const uint4 u = *reinterpret_cast<const uint4 *>(child + 8 * p);
         const uint4 v = *reinterpret_cast<const uint4 *>(child + 8 * p + 4);
-        if (at + p < a.words) a.flags[at + p] = u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w;
+        a.flags[at + p] = u.x | u.y | u.z | u.w | v.x | v.y | v.z | v.w;
       }
       child = a.flags + at;
       __syncthreads();

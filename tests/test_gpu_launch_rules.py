@@ -81,6 +81,20 @@ def test_brick_build_lists(n, fill, dtype, planned):
         assert torch.equal(vct.read_level(dense, l), vct.read_level(bricks, l)), l
 
 
+# Pyramids cut off inside their bricked levels (n = 128 has four, n = 256 takes
+# the scan of several CTAs).
+@pytest.mark.parametrize("n,levels", [(16, 1), (64, 1), (64, 2), (128, 1), (128, 3), (128, 4),
+                                      (256, 1), (256, 4)])
+def test_brick_build_few_levels(n, levels):
+    g = torch.rand((n, n, n, 4), device="cuda")
+    g[: n // 2] = 0
+    dense = vct.build_mips(g, levels=levels)
+    bricks = vct.build_mips(g, levels=levels, layout="bricks")
+    vct.pyramid_status(bricks)
+    for l in range(levels):
+        assert torch.equal(vct.read_level(dense, l), vct.read_level(bricks, l)), l
+
+
 def test_planned_build_checks_its_pool_and_scratch():
     lib, abi = vct.lib(), vct._abi
     g = torch.rand((64, 64, 64, 4), device="cuda")
