@@ -336,7 +336,8 @@ typedef struct {
 typedef struct {
   int32_t tile_w, tile_h;   /* pixels per work item (queue granularity)      */
   int32_t lanes_per_pixel;  /* 1, 2, 4 or 8 lanes share one pixel's cones    */
-  int32_t ctas_per_sm;      /* persistent CTAs per SM; 0 = occupancy limit   */
+  int32_t ctas_per_sm;      /* persistent CTAs of 256 threads per SM; 0 = the
+                               library's CTA size and as many as fit         */
 } vct_launch_config;
 
 /* Per-call counters left in the trace workspace (device memory). */

@@ -678,9 +678,11 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
                   "vct_trace: views of one call must use pyramids of one dtype, and all or "
                   "none anisotropic");
     L->n_views = nv;
-    int grid = std::max(1, std::min(cursor, per_sm * sms)), threads = kFwdThreads;
+    // An explicit count is of CTAs of kExplicitThreads.
+    int threads = cfg.ctas_per_sm == 0 ? kFwdThreads : kExplicitThreads;
+    int grid = std::max(1, std::min(cursor, per_sm * sms));
     // about two waves of the launch's warps, in small tiles, at the end
-    const int64_t tail_px = (int64_t)2 * grid * (kFwdThreads / 32) * kSmallTileW * kSmallTileH;
+    const int64_t tail_px = (int64_t)2 * grid * (threads / 32) * kSmallTileW * kSmallTileH;
     if (L->group) {
       L->total_tiles = L->n_big = cursor;
       const int per_cta = kSplitThreads / 32 / L->group;  // tiles a CTA takes at a time

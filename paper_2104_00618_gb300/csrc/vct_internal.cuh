@@ -26,6 +26,8 @@ constexpr int kTraceThreads = 256;      // CTA shape of the adjoint trace kernel
 #endif
 constexpr int kFwdThreads = VCT_FWD_THREADS;
 constexpr int kTraceMinBlocks = VCT_TRACE_MIN_BLOCKS;
+// CTAs of a launch whose caller says how many an SM gets (two fit).
+constexpr int kExplicitThreads = 256;
 // CTAs of small launches, whose warps share tiles: as many warps per SM in two
 // CTAs, so that fewer tiles than that spread over more SMs.
 constexpr int kSplitThreads = 256, kSplitBlocks = 2;

@@ -203,13 +203,48 @@ def test_forward_shapes(w, h, spec, occ, nd, rough, dtype, layout, flags):
             assert (x - y).abs().max() <= 32 * 2.0 ** -24 * max(1.0, float(y.abs().max()))
 
 
-# Tiles of 192 pixels and more of dense float32 frames run in two CTAs of half
-# the size per SM, just below that in one; an explicit CTA count keeps one.
-# The same pixels in the same warps' order: the same bits.  Eight pyramids
-# take the most shared memory.
+class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v1
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3),
+                ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p)]
+
+
+def _launch(P, view, prm, cfg=None):
+    """(CTAs, threads per CTA, work-queue cursor afterwards) of a trace's one
+    kernel.  The cursor counts the items and one last pull by every warp (or
+    group of warps), so it tells tiles apart."""
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        vct.trace(P, view, prm, cfg=cfg, workspace=ws)
+    drv = ctypes.CDLL("libcuda.so.1")
+    raw = ctypes.c_void_p(graph.raw_cuda_graph())
+    count = ctypes.c_size_t()
+    assert drv.cuGraphGetNodes(raw, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert drv.cuGraphGetNodes(raw, nodes, ctypes.byref(count)) == 0
+    kernels = []
+    for node in nodes:
+        kind = ctypes.c_int()
+        assert drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 0:  # a kernel
+            k = _KernelNode()
+            assert drv.cuGraphKernelNodeGetParams(ctypes.c_void_p(node), ctypes.byref(k)) == 0
+            kernels.append(k)
+    assert len(kernels) == 1
+    graph.replay()
+    queue = int(ws[:56].cpu().numpy().view(np.uint32)[12])
+    return kernels[0].grid[0], kernels[0].block[0], queue
+
+
+# Tiles of 192 pixels and more of dense float32 frames run in two CTAs of 256
+# threads per SM, just below that in one of 512; an explicit CTA count is one
+# of CTAs of 256.  The same pixels in the same warps' order: the same bits.
+# Eight pyramids take the most shared memory.
 @pytest.mark.parametrize("tile,views", [((8, 24), 1), ((16, 16), 1), ((8, 23), 1), ((12, 16), 8)])
 def test_forward_cta_sizes(tile, views):
     w, h = 1001, 701
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
     rng = np.random.default_rng(views)
     scene = vs.box_scene(16, 4, 5, room=True)
     dirs, wts = vs.cone_table_ring6()
@@ -218,16 +253,25 @@ def test_forward_cta_sizes(tile, views):
     P = [vct.build_mips(torch.from_numpy(scene["grid"]).cuda()) for _ in range(views)]
     host = vs.interior_view(scene, w, h, rng, with_roughness=True)
     out = []
-    for per_sm in (0, 1):
+    for per_sm in (0, 1, 2):
         v = [vct.View.from_host({**host, "pyramid": i}) for i in range(views)]
-        stats = vct.read_stats(vct.trace(P, v, prm, cfg=vct.launch_config(*tile, 1, per_sm)))
+        cfg = vct.launch_config(*tile, 1, per_sm)
+        ctas, threads, _ = _launch(P, v, prm, cfg)
+        if per_sm:
+            assert (ctas, threads) == (per_sm * sms, 256)
+        else:
+            assert (ctas, threads) == ((2 * sms, 256) if tile[0] * tile[1] >= 192 else (sms, 512))
+        for x in v:
+            x.alloc_outputs()
+        stats = vct.read_stats(vct.trace(P, v, prm, cfg=cfg))
         out.append((v, stats))
-    (a, sa), (b, sb) = out
-    assert sa == sb
-    for x, y in zip(a, b):
-        assert torch.equal(x.out_diffuse, y.out_diffuse)
-        assert torch.equal(x.out_specular, y.out_specular)
-        assert torch.equal(x.out_visibility, y.out_visibility)
+    (a, sa) = out[0]
+    for b, sb in out[1:]:
+        assert sa == sb
+        for x, y in zip(a, b):
+            assert torch.equal(x.out_diffuse, y.out_diffuse)
+            assert torch.equal(x.out_specular, y.out_specular)
+            assert torch.equal(x.out_visibility, y.out_visibility)
 
 
 # Four, five and all eight pyramids of a call: from five up the step tables
@@ -280,40 +324,6 @@ def test_large_build_paths_agree(levels, dtype):
     b = vct.build_mips(shifted.clone(), levels=levels, dtype=dtype)
     for l in range(levels):
         assert torch.equal(vct.read_level(a, l), vct.read_level(b, l)), l
-
-
-class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v1
-    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3),
-                ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
-                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p)]
-
-
-def _launch(P, view, prm, cfg=None):
-    """(CTAs, threads per CTA, work-queue cursor afterwards) of a trace's one
-    kernel.  The cursor counts the items and one last pull by every warp (or
-    group of warps), so it tells tiles apart."""
-    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
-    graph = torch.cuda.CUDAGraph(keep_graph=True)
-    with torch.cuda.graph(graph):
-        vct.trace(P, view, prm, cfg=cfg, workspace=ws)
-    drv = ctypes.CDLL("libcuda.so.1")
-    raw = ctypes.c_void_p(graph.raw_cuda_graph())
-    count = ctypes.c_size_t()
-    assert drv.cuGraphGetNodes(raw, None, ctypes.byref(count)) == 0
-    nodes = (ctypes.c_void_p * count.value)()
-    assert drv.cuGraphGetNodes(raw, nodes, ctypes.byref(count)) == 0
-    kernels = []
-    for node in nodes:
-        kind = ctypes.c_int()
-        assert drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
-        if kind.value == 0:  # a kernel
-            k = _KernelNode()
-            assert drv.cuGraphKernelNodeGetParams(ctypes.c_void_p(node), ctypes.byref(k)) == 0
-            kernels.append(k)
-    assert len(kernels) == 1
-    graph.replay()
-    queue = int(ws[:56].cpu().numpy().view(np.uint32)[12])
-    return kernels[0].grid[0], kernels[0].block[0], queue
 
 
 # Tuning never leaves a call slower than the library's own pick: not the call
