@@ -379,30 +379,31 @@ int64_t total_pixels(const vct_view *views, int32_t n_views) {
 }
 
 // Tile of a launch that the caller gives no shape for.  Where the specular
-// aperture follows the roughness, a larger tile sorts more cones by length;
-// a smaller one leaves less idle in the last wave of warps.  Measured (9 + 1
-// + 1 cones, 256^3), 8 x 8 / 8 x 16 / 8 x 24 / 16 x 16: 0.41 M pixels 1671 /
-// 1598 / - / 2049 us, 0.92 M 3189 / 2994 / 3088 / 3131, 1.44 M (means of eight
-// scenes) 4583 / 4286 / 4238 / 4467, 2.07 M 6480 / 6015 / 5980 / 6141 (binary16
-// 7034 / 6517 / 6461 / 6644), 3.69 M 12467 / 11544 / - / 11082 (all with one
-// CTA per SM; with two, as dense float32 takes for the last two tiles, 1.44 M
-// 4315 / 4365 / 4371 without the first, 2.07 M 6082 / 6017 / 6068); one aperture
-// (6 + 1 cones, 64^3): 0.52 M 656 / 704 / - / 804, 2.07 M 2373 / 2398 / - / 2596.
-vct_launch_config default_cfg(const vct_pyramid *pyrs, const vct_view *views, int32_t n_views,
-                              const vct_trace_params &P) {
+// aperture follows the roughness, a larger tile sorts more cones by length; a
+// smaller one leaves less idle in the last wave of warps, so the lines lie at
+// pixels per warp of a full chip (16 per SM).  Measured (9 + 1 + 1 cones, 256^3
+// and 512^3, mean of four rooms of filled boxes and four views of surface
+// shells, us), 8 x 16 / 8 x 24 / 16 x 16, on 152 SMs:
+//   pixels       float32                 binary16
+//   0.80 M    2728 /  2693 /  2880    3308 /  3426 /  3623
+//   1.08 M    3482 /  3502 /  3490    4258 /  4156 /  4535
+//   1.44 M    4615 /  4705 /  4642    5612 /  5521 /  5729
+//   2.07 M    6493 /  6502 /  6527    7925 /  7809 /  7856
+//   2.62 M    8094 /  8046 /  8093    9889 /  9694 /  9534
+//   2.95 M    9106 /  9083 /  8905   11128 / 10944 / 10886
+//   3.69 M   11285 / 11132 / 11073   13786 / 13432 / 13357
+// (float32 in 8 x 24 and 16 x 16 with two CTAs per SM, as the launch takes it).
+// One aperture (6 + 1 cones, 64^3), 8 x 8 / 8 x 16 / 16 x 16: 0.52 M 656 / 704 /
+// 804, 2.07 M 2373 / 2398 / 2596.
+vct_launch_config default_cfg(const vct_view *views, int32_t n_views, const vct_trace_params &P) {
   bool rough = false;
   for (int i = 0; i < n_views; ++i) rough |= views[i].roughness != nullptr;
   if (!P.spec_enable || !rough || P.spec_aperture_min == P.spec_aperture_max)
     return vct_launch_config{8, 8, 1, 0};
+  const int64_t warps = (int64_t)sm_count() * (kFwdThreads / 32);
   const int64_t pixels = total_pixels(views, n_views);
-  if (pixels < 1000000) return vct_launch_config{8, 16, 1, 0};
-  // (dense float32 at 1.44 M, two CTAs: 8 x 24 5.40 ms, 16 x 16 5.30 in a room
-  // of surface shells, 4365 and 4371 us as above; at 2.07 M 7.37 - 7.49 and
-  // 7.36 - 7.57 ms, 6017 and 6068 us)
-  const vct_pyramid &p0 = pyrs[views[0].pyramid];
-  const int64_t lower = p0.dtype == VCT_F32 && p0.layout == VCT_LAYOUT_DENSE && !P.flags ? 1750000 : 0;
-  return pixels >= lower && pixels < 3000000 ? vct_launch_config{8, 24, 1, 0}
-                                             : vct_launch_config{16, 16, 1, 0};
+  if (pixels < 400 * warps) return vct_launch_config{8, 16, 1, 0};
+  return pixels < 1000 * warps ? vct_launch_config{8, 24, 1, 0} : vct_launch_config{16, 16, 1, 0};
 }
 
 vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs,
@@ -413,7 +414,7 @@ vct_launch_config pick_cfg(const vct_launch_config *cfg, const vct_pyramid *pyrs
   std::lock_guard<std::mutex> g(g_tune_mu);
   auto it = g_tuned.find(tune_key(pyrs, views, n_views, P));
   tuned = it != g_tuned.end();
-  return tuned ? it->second : default_cfg(pyrs, views, n_views, *P);
+  return tuned ? it->second : default_cfg(views, n_views, *P);
 }
 
 struct TraceStatsLayout {
@@ -782,7 +783,7 @@ vct_status vct_autotune_trace(const vct_pyramid *pyrs, int32_t n_pyr, const vct_
   const int lpps[4] = {1, 2, 4, 8};
   float own_ms = 0.f, best_ms = 1e30f;
   vct_launch_config bc{16, 16, 1, 0};
-  st = timed(default_cfg(pyrs, views, n_views, *params), true, own_ms);
+  st = timed(default_cfg(views, n_views, *params), true, own_ms);
   for (int i = 0; st == VCT_OK && i < 20; ++i) {
     const vct_launch_config c{tiles[i / 4][0], tiles[i / 4][1], lpps[i % 4], 0};
     float ms = 0.f;

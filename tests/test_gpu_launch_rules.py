@@ -274,6 +274,36 @@ def test_forward_cta_sizes(tile, views):
             assert torch.equal(x.out_visibility, y.out_visibility)
 
 
+# The default tile where the specular aperture follows the roughness: 8 x 16
+# below 400 pixels per warp of a full chip, 8 x 24 below 1000, 16 x 16 from
+# there; each side of both lines, against the same launch with that shape given
+# and the pixels of another.  (A view as wide as the chip has warps.)
+@pytest.mark.parametrize("h,tile", [(399, (8, 16)), (400, (8, 24)), (999, (8, 24)),
+                                    (1000, (16, 16))])
+@pytest.mark.parametrize("dtype,layout,flags", [("f32", "dense", 0), ("f16", "dense", 0),
+                                                ("f32", "bricks", 8)])
+def test_default_tiles(h, tile, dtype, layout, flags):
+    w = 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    scene = vs.box_scene(16, 4, 5, room=True)
+    dirs, wts = vs.cone_table_ring6()
+    prm = vs.trace_params(dirs[:2], wts[:2], 1.0, spec_enable=1, spec_aperture_min=0.3,
+                          spec_aperture_max=0.9, occ_enable=1, light=scene["light"])
+    prm = vs.variant_params(prm, flags)
+    part = vs.interior_view(scene, w // 8, h, np.random.default_rng(h), with_roughness=True)
+    host = {**part, "width": w}
+    for k in ("position", "normal", "roughness", "mask"):
+        a = np.asarray(part[k])
+        host[k] = np.tile(a.reshape(h, w // 8, -1), (1, 8, 1)).reshape(-1)
+    P = vct.build_mips(torch.from_numpy(scene["grid"]).cuda(), dtype=dtype, layout=layout)
+    v = vct.View.from_host(host)
+    assert _launch(P, v, prm) == _launch(P, v, prm, vct.launch_config(*tile))
+    own = (v.out_diffuse.clone(), v.out_specular.clone(), v.out_visibility.clone())
+    vct.trace(P, v, prm, cfg=vct.launch_config(16, 8))
+    assert torch.equal(v.out_diffuse, own[0])
+    assert torch.equal(v.out_specular, own[1])
+    assert torch.equal(v.out_visibility, own[2])
+
+
 # Four, five and all eight pyramids of a call: from five up the step tables
 # pass the shared memory of a plain launch.  Each view alone gives the same
 # bits.
