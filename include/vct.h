@@ -373,6 +373,9 @@ size_t vct_trace_workspace_bytes(void);
  * [0, levels-1]; trilinear at floor(lambda) and floor(lambda)+1, linear in
  * frac(lambda); colour c += (1 - alpha) a_s c_s, alpha += (1 - alpha) a_s;
  * float32 arithmetic throughout (FP16 pyramids are widened on load).
+ * With lanes_per_pixel 1, as in every shape the library picks by itself, a
+ * pixel's outputs have the same bits whatever the tile, the number of pixels
+ * and the other views of the call; more lanes add D's cones in another order.
  * Errors: VCT_ERR_INVALID_ARG (NULL pointers where required, bad shapes or
  * parameters, pyramid index out of range), VCT_ERR_WORKSPACE, VCT_ERR_CUDA.
  */

@@ -399,9 +399,11 @@ __global__ void __launch_bounds__(kFwdThreads, kTraceMinBlocks) trace_kernel(con
 // Small launches: the warps of a group (L.group, 2 or 4) share a tile of 8 x 4
 // pixels, one pixel per lane, and split its cones: the first warp marches the
 // specular cone, the longest, the others the rest in turn (all of them,
-// without a specular cone).  Each warp leaves its part of D in shared memory
-// and the second warp sums the parts and writes the pixel.  The lanes of a
-// warp still march one cone in lock step.
+// without a specular cone).  Each warp leaves its cones' results in shared
+// memory; the second warp sums the diffuse ones in the order of the cones, as
+// one lane does in trace_kernel (so a pixel's bits do not depend on how many
+// pixels its call has), and writes the pixel.  The lanes of a warp still march
+// one cone in lock step.
 __device__ __forceinline__ void group_sync(int id, int threads) {
   __syncwarp();  // (the barrier wants whole warps)
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
@@ -417,10 +419,13 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
   const int n_cones = L.n_diffuse + L.spec_enable + L.occ_enable;
   const float T0 = L.spec.t0_vox;
   __shared__ uint2 s_lut[kSpreadLut];
-  __shared__ float4 s_part[kWarps][32];  // a warp's part of D; the specular warp's S
-  __shared__ float s_vis[kWarps][32];    // transmittance of the occlusion cone
-  __shared__ int s_item[kWarps];
+  __shared__ float4 s_spec[kWarps / 2][32];  // per group and pixel: S,
+  __shared__ float s_vis[kWarps / 2][32];    // transmittance of the occlusion cone
+  __shared__ int s_item[kWarps / 2];
+  // n_pyr * 2 * kStepTab entries, then the diffuse cones' results per group,
+  // cone and pixel
   extern __shared__ __align__(16) float4 s_tab[];
+  float4 *s_diff = s_tab + L.n_pyr * 2 * kStepTab + group * L.n_diffuse * 32 + lane;
   fill_step_table(s_tab, L.pyr, L.n_pyr, T0);
   fill_spread_lut(s_lut);  // (its barrier also covers s_tab)
 
@@ -438,8 +443,6 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
     const bool inimg = px < V.W && py < V.H;
     const int p = py * V.W + px;
     const bool active = inimg && (V.mask == nullptr || V.mask[p] != 0);
-    float4 D = make_float4(0.f, 0.f, 0.f, 0.f);
-    float vis = 0.f;
     if (active) {
       float x[3], n[3];
 #pragma unroll
@@ -487,13 +490,9 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
         n_cone[cs.kind] += 1u;
         if (V.state) V.state[(size_t)c * V.W * V.H + p] = cst;
         if (cs.kind == kDiffuse) {
-          const float wt = L.diffuse_weight[cs.diffuse_index];
-          D.x = fmaf(wt, r.x, D.x);
-          D.y = fmaf(wt, r.y, D.y);
-          D.z = fmaf(wt, r.z, D.z);
-          D.w = fmaf(wt, r.w, D.w);
+          s_diff[cs.diffuse_index * 32] = r;
         } else if (cs.kind == kOcclusion) {
-          vis = trans;
+          s_vis[group][lane] = trans;
         } else {
           if constexpr (kVar) {
             if (L.var.flags & VCT_FLAG_SPEC_GRACE) {
@@ -503,35 +502,26 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
               r.z *= f;
             }
           }
-          D = r;  // (this warp has no other cone)
+          s_spec[group][lane] = r;
         }
       }
     }
-    s_part[warp][lane] = D;
-    s_vis[warp][lane] = vis;
     group_sync(bar, bar_threads);
     if (q == 1 && inimg) {
-      const int w0 = group * L.group;
-      float4 S = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (L.spec_enable) {
-        S = s_part[w0][lane];
-      } else {
-        const float4 o = s_part[w0][lane];
-        D.x += o.x;
-        D.y += o.y;
-        D.z += o.z;
-        D.w += o.w;
-        vis += s_vis[w0][lane];
+      float4 D = make_float4(0.f, 0.f, 0.f, 0.f), S = D;
+      float vis = 1.0f;
+      if (active) {
+        for (int k = 0; k < L.n_diffuse; ++k) {
+          const float4 r = s_diff[k * 32];
+          const float wt = L.diffuse_weight[k];
+          D.x = fmaf(wt, r.x, D.x);
+          D.y = fmaf(wt, r.y, D.y);
+          D.z = fmaf(wt, r.z, D.z);
+          D.w = fmaf(wt, r.w, D.w);
+        }
+        if (L.spec_enable) S = s_spec[group][lane];
+        if (L.occ_enable) vis = s_vis[group][lane];
       }
-      for (int k = 2; k < L.group; ++k) {
-        const float4 o = s_part[w0 + k][lane];
-        D.x += o.x;
-        D.y += o.y;
-        D.z += o.z;
-        D.w += o.w;
-        vis += s_vis[w0 + k][lane];
-      }
-      if (!(L.occ_enable && active)) vis = 1.0f;
       if (V.outD) reinterpret_cast<float4 *>(V.outD)[p] = D;
       if (V.outS) reinterpret_cast<float4 *>(V.outS)[p] = S;
       if (V.outV) V.outV[p] = vis;
@@ -543,7 +533,7 @@ __global__ void __launch_bounds__(kSplitThreads, kSplitBlocks)
         }
       }
     }
-    // (the next item's barrier orders the parts' reads with their next writes)
+    // (the next item's barrier orders the results' reads with their next writes)
   }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -562,16 +552,21 @@ inline size_t step_table_bytes(int n_pyr) { return (size_t)n_pyr * 2 * kStepTab 
 // and the sort keys of its warps, behind them (trace_kernel).
 inline size_t sort_key_bytes(int threads) { return (size_t)threads / 32 * kMaxSortPixels * 4; }
 
-// Static shared memory of trace_kernel.  With the tables of five pyramids and
-// more a CTA passes the 48 KB of a plain launch; the limit asked for is always
-// that of VCT_MAX_PYRAMIDS, so that callers on other threads do not lower it.
-constexpr size_t kTraceStatic = kSpreadLut * sizeof(uint2);
+// and the diffuse results of the tiles its groups hold (trace_split_kernel).
+inline size_t split_bytes(int group, int n_diffuse) {
+  return group ? (size_t)(kSplitThreads / 32 / group) * n_diffuse * 32 * sizeof(float4) : 0;
+}
+
+// Static shared memory of the two kernels (rounded up).  Where a CTA passes the
+// 48 KB of a plain launch, the limit asked for is always the largest any launch
+// takes, so that callers on other threads do not lower it.
+constexpr size_t kTraceStatic = kSpreadLut * sizeof(uint2) + 4096;
 
 template <typename K>
-cudaError_t allow_shared(K kernel, size_t dyn) {
+cudaError_t allow_shared(K kernel, size_t dyn, size_t most) {
   if (kTraceStatic + dyn <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(step_table_bytes(VCT_MAX_PYRAMIDS) + sort_key_bytes(kFwdThreads)));
+                              (int)(step_table_bytes(VCT_MAX_PYRAMIDS) + most));
 }
 
 template <int LPP, int DT, bool BR, bool AN = false>
@@ -579,21 +574,19 @@ cudaError_t launch_t(const TraceLaunch &L, int grid, int threads, cudaStream_t s
   const size_t dyn = step_table_bytes(L.n_pyr);
   if constexpr (LPP == 1) {
     if (L.group) {
-      if (L.var.flags)
-        trace_split_kernel<DT, true, BR, AN><<<grid, threads, dyn, s>>>(L);
-      else
-        trace_split_kernel<DT, false, BR, AN><<<grid, threads, dyn, s>>>(L);
+      auto kernel = L.var.flags ? trace_split_kernel<DT, true, BR, AN>
+                                : trace_split_kernel<DT, false, BR, AN>;
+      const size_t all = dyn + split_bytes(L.group, L.n_diffuse);
+      if (cudaError_t e = allow_shared(kernel, all, split_bytes(2, VCT_MAX_DIFFUSE))) return e;
+      kernel<<<grid, threads, all, s>>>(L);
       return cudaGetLastError();
     }
   }
+  auto kernel = L.var.flags ? trace_kernel<LPP, DT, true, BR, AN>
+                            : trace_kernel<LPP, DT, false, BR, AN>;
   const size_t all = dyn + sort_key_bytes(threads);
-  if (L.var.flags) {
-    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, true, BR, AN>, all)) return e;
-    trace_kernel<LPP, DT, true, BR, AN><<<grid, threads, all, s>>>(L);
-  } else {
-    if (cudaError_t e = allow_shared(trace_kernel<LPP, DT, false, BR, AN>, all)) return e;
-    trace_kernel<LPP, DT, false, BR, AN><<<grid, threads, all, s>>>(L);
-  }
+  if (cudaError_t e = allow_shared(kernel, all, sort_key_bytes(kFwdThreads))) return e;
+  kernel<<<grid, threads, all, s>>>(L);
   return cudaGetLastError();
 }
 

@@ -1,7 +1,6 @@
-"""Launch rules picked by size: each side of a rule against the FP64 oracle.
-
-A pixel's sums are the same terms in another order on either side, so every
-case is held to the float32 bound of the repository's other comparisons.
+"""Launch rules picked by size: each side of a rule, bit for bit against another
+launch shape or, for the adjoint's float atomics, against the FP64 oracle within
+the float32 bound of the repository's other comparisons.
 """
 import ctypes
 
@@ -161,48 +160,6 @@ def test_planned_build_refuses_other_plans(case, dtype):
                               rtol=1e-5 if dtype == "f32" else 2e-3)
 
 
-# A launch without a shape shares a tile's cones among 4 warps (up to 608
-# tiles of 8 x 4 pixels on 152 SMs), 2 (up to 4864) or none, where the tile
-# depends on the roughness; each against one warp per 8 x 8 tile: the cones
-# march the same steps (states bit for bit), D sums the same cones in another
-# order (at most 32 terms, 2^-24 each).
-@pytest.mark.parametrize("w,h,spec,occ,nd,rough", [
-    (1, 1, 1, 1, 6, False), (9, 5, 0, 1, 1, False), (37, 21, 1, 0, 2, True), (64, 33, 0, 0, 5, False),
-    (160, 121, 1, 1, 6, True), (160, 125, 1, 1, 6, True), (400, 389, 1, 1, 1, False),
-    (400, 393, 1, 1, 1, False), (500, 400, 1, 0, 1, True), (300, 200, 1, 0, 0, True)])
-@pytest.mark.parametrize("dtype,layout,flags", [("f32", "dense", 0), ("f16", "bricks", 0),
-                                                ("f32", "aniso", 0), ("f32", "dense", 15),
-                                                ("f32", "dense", 32 + 24)])
-def test_forward_shapes(w, h, spec, occ, nd, rough, dtype, layout, flags):
-    n = 16
-    rng = np.random.default_rng(w + h)
-    scene = vs.box_scene(n, 4, 5, room=True)
-    view = vs.interior_view(scene, w, h, rng, with_roughness=rough)
-    view["mask"] = (rng.random(w * h) >= 0.1).astype(np.uint8)
-    dirs, wts = vs.cone_table_ring6()
-    prm = vs.trace_params(dirs[:nd], wts[:nd], 1.0, spec_enable=spec, spec_aperture_min=0.3,
-                          spec_aperture_max=0.9, occ_enable=occ, light=scene["light"])
-    prm = vs.variant_params(prm, flags)
-    P = vct.build_mips(torch.from_numpy(scene["grid"]).cuda(), dtype=dtype, layout=layout)
-    out = []
-    for cfg in (None, vct.launch_config(8, 8, 1)):
-        v = vct.View.from_host(view)
-        if flags & vct.FLAG_SHADE:
-            v.albedo = torch.full((w * h, 3), 0.7, device="cuda")
-            v.alloc_outputs(radiance=True)
-        v.alloc_cone_state(prm).cone_state.zero_()
-        stats = vct.read_stats(vct.trace(P, v, prm, cfg=cfg))
-        out.append((v, stats))
-    (a, sa), (b, sb) = out
-    assert sa == sb
-    assert torch.equal(a.cone_state, b.cone_state)
-    assert torch.equal(a.out_specular, b.out_specular)
-    assert torch.equal(a.out_visibility, b.out_visibility)
-    for x, y in ((a.out_diffuse, b.out_diffuse), (a.out_radiance, b.out_radiance)):
-        if x is not None:
-            assert (x - y).abs().max() <= 32 * 2.0 ** -24 * max(1.0, float(y.abs().max()))
-
-
 class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v1
     _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3),
                 ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
@@ -235,6 +192,58 @@ def _launch(P, view, prm, cfg=None):
     graph.replay()
     queue = int(ws[:56].cpu().numpy().view(np.uint32)[12])
     return kernels[0].grid[0], kernels[0].block[0], queue
+
+
+# A launch without a shape shares a tile's cones among 4 warps (up to 4 tiles of
+# 8 x 4 pixels per SM, three cones and more besides the specular one), 2 (up to
+# 32 per SM, two cones and more) or none; widths below 0 are multiples of the
+# SM count, heights then on a limit and just above it.  Each against one warp
+# per 16 x 8 tile: the cones march the same steps and D sums them in the same
+# order, so every output has the same bits.
+@pytest.mark.parametrize("w,h,spec,occ,nd,rough,warps", [
+    (1, 1, 1, 1, 6, False, 4), (9, 5, 0, 1, 1, False, 2), (37, 21, 1, 0, 2, True, 2),
+    (64, 33, 0, 0, 5, False, 4), (60, 40, 1, 1, 32, False, 4), (160, 121, 1, 1, 32, True, 2),
+    (-8, 16, 1, 1, 6, True, 4), (-8, 17, 1, 1, 6, True, 2), (-8, 16, 0, 1, 6, False, 4),
+    (-8, 128, 1, 1, 1, True, 2), (-8, 129, 1, 1, 1, True, 0), (-8, 128, 0, 1, 2, False, 2),
+    (-8, 129, 0, 1, 2, False, 0), (300, 200, 1, 0, 0, True, 0)])
+@pytest.mark.parametrize("dtype,layout,flags", [("f32", "dense", 0), ("f16", "bricks", 0),
+                                                ("f32", "aniso", 0), ("f32", "dense", 15),
+                                                ("f32", "dense", 32 + 24)])
+def test_forward_shapes(w, h, spec, occ, nd, rough, warps, dtype, layout, flags):
+    n = 16
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = w if w > 0 else -w * sms
+    rng = np.random.default_rng(w + h)
+    scene = vs.box_scene(n, 4, 5, room=True)
+    view = vs.interior_view(scene, w, h, rng, with_roughness=rough)
+    view["mask"] = (rng.random(w * h) >= 0.1).astype(np.uint8)
+    dirs, wts = vs.cone_table_ring6()
+    dirs, wts = np.tile(dirs, (6, 1)), np.tile(wts, 6) / 6
+    prm = vs.trace_params(dirs[:nd], wts[:nd], 1.0, spec_enable=spec, spec_aperture_min=0.3,
+                          spec_aperture_max=0.9, occ_enable=occ, light=scene["light"])
+    prm = vs.variant_params(prm, flags)
+    P = vct.build_mips(torch.from_numpy(scene["grid"]).cuda(), dtype=dtype, layout=layout)
+    out = []
+    for cfg in (None, vct.launch_config(16, 8, 1)):
+        v = vct.View.from_host(view)
+        if flags & vct.FLAG_SHADE:
+            v.albedo = torch.full((w * h, 3), 0.7, device="cuda")
+            v.alloc_outputs(radiance=True)
+        if cfg is None:
+            tiles = -(-w // 8) * -(-h // 4)
+            shared = (min(-(-tiles * warps // 8), 2 * sms), 256) if warps else None
+            own = _launch(P, v, prm)
+            assert own[:2] == shared if warps else own == _launch(
+                P, v, prm, vct.launch_config(8, 16 if rough and spec else 8))
+        v.alloc_cone_state(prm).cone_state.zero_()
+        stats = vct.read_stats(vct.trace(P, v, prm, cfg=cfg))
+        out.append((v, stats))
+    (a, sa), (b, sb) = out
+    assert sa == sb
+    assert torch.equal(a.cone_state, b.cone_state)
+    for x, y in ((a.out_diffuse, b.out_diffuse), (a.out_specular, b.out_specular),
+                 (a.out_visibility, b.out_visibility), (a.out_radiance, b.out_radiance)):
+        assert x is None or torch.equal(x, y)
 
 
 # Tiles of 192 pixels and more of dense float32 frames run in two CTAs of 256
@@ -306,7 +315,7 @@ def test_default_tiles(h, tile, dtype, layout, flags):
 
 # Four, five and all eight pyramids of a call: from five up the step tables
 # pass the shared memory of a plain launch.  Each view alone gives the same
-# bits.
+# bits, in the default shape (whose warps share tiles here) as in a given one.
 @pytest.mark.parametrize("n_pyr", [4, 5, 8])
 @pytest.mark.parametrize("lpp,cfg", [(1, True), (1, False), (4, True)])
 @pytest.mark.parametrize("layout,flags", [("dense", 0), ("bricks", 0), ("aniso", 0), ("dense", 15)])
@@ -336,8 +345,7 @@ def test_many_pyramids(n_pyr, lpp, cfg, layout, flags):
         vct.trace([P[i]], [one], prm, cfg=shape or vct.launch_config(8, 8, 1))
         assert torch.equal(got[i].out_specular, one.out_specular)
         assert torch.equal(got[i].out_visibility, one.out_visibility)
-        d = (got[i].out_diffuse - one.out_diffuse).abs().max()
-        assert d <= (0 if cfg else 32 * 2.0 ** -24 * max(1.0, float(one.out_diffuse.abs().max())))
+        assert torch.equal(got[i].out_diffuse, one.out_diffuse)
 
 
 # Sizes whose level 4 passes one tail CTA's 4096 texels, whole and cut off
