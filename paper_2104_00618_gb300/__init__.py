@@ -153,7 +153,8 @@ def build_mips(level0: torch.Tensor, levels: int | None = None, dtype="f32",
                                            scratch.numel(), _stream(stream)),
               "vct_build_mips_planned")
         if stream is not None:
-            scratch.record_stream(stream)  # allocated on the current stream
+            # (allocated on the current stream; `stream` may be any handle holder)
+            scratch.record_stream(torch.cuda.ExternalStream(_stream(stream), level0.device))
         return pyr
     pyr = out if out is not None else Pyramid(n, levels, dtype, origin, size, level0.device,
                                               layout)

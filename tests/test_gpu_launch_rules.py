@@ -94,6 +94,22 @@ def test_brick_build_few_levels(n, levels):
         assert torch.equal(vct.read_level(dense, l), vct.read_level(bricks, l)), l
 
 
+# A stream is anything with a cuda_stream handle, here as in every other call.
+def test_brick_build_takes_a_stream_handle():
+    class Handle:
+        def __init__(self, stream):
+            self.cuda_stream = stream.cuda_stream
+
+    g = torch.rand((32, 32, 32, 4), device="cuda")
+    want = vct.read_level(vct.build_mips(g, layout="bricks"), 1)
+    torch.cuda.synchronize()
+    for side in (torch.cuda.Stream(), torch.cuda.default_stream()):
+        for stream in (side, Handle(side)):
+            P = vct.build_mips(g, layout="bricks", stream=stream)
+            side.synchronize()
+            assert torch.equal(vct.read_level(P, 1), want)
+
+
 def test_planned_build_checks_its_pool_and_scratch():
     lib, abi = vct.lib(), vct._abi
     g = torch.rand((64, 64, 64, 4), device="cuda")
