@@ -22,8 +22,9 @@ struct TableArgs {
 // One warp per level-0 brick: where any channel of its 512 texels is
 // non-zero, the brick and the bricks above it in every bricked level are
 // flagged (the flags start at 0; warps that share a coarser brick store the
-// same 1); `small`: each level-0 flag is written, 0 or 1, and no other.  level0 is dense [z][y][x][4]; the brick's rows of 8 texels are 128
-// bytes.  512^3: 0.32 ms for 2.15 GB, the HBM copy rate.
+// same 1); `small`: each level-0 flag is written, 0 or 1, and no other.  level0
+// is dense [z][y][x][4]; the brick's rows of 8 texels are 128 bytes.  512^3:
+// 0.32 ms for 2.15 GB, the HBM copy rate.
 __global__ void __launch_bounds__(256) occupancy_kernel(const float4 *level0, int n,
                                                         const __grid_constant__ TableArgs a,
                                                         bool small) {
@@ -51,9 +52,9 @@ __global__ void __launch_bounds__(256) occupancy_kernel(const float4 *level0, in
 
 // Flags -> slots, by an exclusive scan over all bricked levels in level order:
 // the tables follow one another without gaps (a level of 64 bricks or more
-// fills 256-byte lines, the last one has 8), so they are scanned as one array.  kScanCtas CTAs take a part each; count_kernel leaves
-// the parts' sums in the header's free words, slots_kernel adds those before
-// its own.  At 512^3 (300 K flags) one CTA alone took 232 us with one flag per
+// fills 256-byte lines, the last one has 8), so they are scanned as one array.
+// kScanCtas CTAs take a part each; count_kernel leaves the parts' sums in the
+// header's free words, slots_kernel adds those before its own.  At 512^3 (300 K flags) one CTA alone took 232 us with one flag per
 // thread and pass, 69 us with 16 (its SM's share of the L2 bandwidth).
 constexpr int kScanThreads = 1024;
 constexpr int kScanRun = 8;    // consecutive flags per thread and pass

@@ -251,9 +251,9 @@ __global__ void __launch_bounds__(256) pack_mips_kernel(const __grid_constant__ 
   int s = 0;
   // This CTA's blocks, kBlockRun at a time.  Of a brick pyramid's only those
   // with an occupied brick are listed (s_list) and read: the texels of the
-  // others are zero, which the empty bricks say already (512^3 room, a fifth
-  // of the blocks occupied: 840 -> 360 us).  Where the pool was too small
-  // every slot is 0 and the blocks are all taken.
+  // others are zero, which the empty bricks say already (512^3 room: 840 -> 285
+  // us, with the slots read ahead and the odd grid below).  Where the pool was
+  // too small every slot is 0 and the blocks are all taken.
   const bool skip = BR && B == 16 && *a.count < a.capacity;  // (and the zero brick)
   for (uint64_t run = blockIdx.x; run < a.nblocks; run += (uint64_t)kBlockRun * gridDim.x) {
     const uint64_t left = (a.nblocks - run + gridDim.x - 1) / gridDim.x;
@@ -389,8 +389,7 @@ __device__ __forceinline__ void wait_for_previous_grid() {
 // four whole level-2 cells and a warp reduces them with shuffles, with no
 // barrier between phases.  The CTA takes 16 units at a time, warp w the w-th
 // and the w+8-th: one phase where X = 256, several phases' where X is smaller.
-// A
-// lane's cell: its 8 children as four 32-byte x pairs (rows of a unit are
+// A lane's cell: its 8 children as four 32-byte x pairs (rows of a unit are
 // 256-byte pieces), written to level 0 at Morton codes 8 code .. 8 code + 7
 // (child jx | jy << 1 | jz << 2, the x pairs contiguous), and their mean to
 // level 1.  The next 16 units' loads are issued as soon as the stores have

@@ -89,8 +89,9 @@ __device__ __forceinline__ void scatter_lane(const BwdLaunch &L, int l, uint32_t
 // against derivative row j % 4, four columns per pair of 16-byte loads, and
 // issues one atomic on a distinct address: contending atomics (the same
 // texel from many lanes) are what makes a naive scatter slow at the coarse
-// levels.  What binds is instruction issue and fixed latencies (ncu: 0.62 of
-// the issue peak, the atomics 3-10 % of the time): this form takes about 80
+// levels.  What binds is instruction issue and fixed latencies (ncu: 0.57 of
+// the issue peak, 0.62 before this form; before it, leaving out the groups'
+// atomics took 3 % off the step, single lanes' 10 %): this form takes about 80
 // instructions per group, where the recursive halving by shuffles that it
 // replaces took 190.  Kernel on 8 views of 512^2, 128^3 grid: 7.70 G -> 6.5 G
 // warp instructions, the whole training step 13.45 -> 12.70 ms; the adjoint
@@ -115,8 +116,9 @@ constexpr int kKeyTotal = VCT_MAX_LEVELS;
 
 template <bool AN>
 __device__ __forceinline__ void scatter_warp(const BwdLaunch &L, const uint32_t *code_off,
-                                             WarpRows &rows, bool act, int l, uint32_t vbase, uint32_t lim,
-                                             const LevelStencil &s, float lw, const float g[4]) {
+                                             WarpRows &rows, bool act, int l, uint32_t vbase,
+                                             uint32_t lim, const LevelStencil &s, float lw,
+                                             const float g[4]) {
   const unsigned full = 0xffffffffu;
   act = act && s.valid != 0u;  // a cell wholly outside the level has nothing to scatter
   if (__ballot_sync(full, act) == 0u) return;
@@ -221,7 +223,8 @@ __device__ __forceinline__ void scatter_warp(const BwdLaunch &L, const uint32_t 
 // forward skipped none (warp-uniform trip count).
 template <bool AN>
 __device__ __forceinline__ void scatter_level(const BwdLaunch &L, const uint32_t *code_off,
-                                              WarpRows &rows, bool act, int l, const LevelStencil &s, float lw,
+                                              WarpRows &rows, bool act, int l,
+                                              const LevelStencil &s, float lw,
                                               const float g[4], const AnisoW &aw) {
   const uint32_t tex = (uint32_t)level_texels(L.pyr.n, l);
   if constexpr (!AN) {
@@ -523,8 +526,8 @@ __global__ void __launch_bounds__(kTraceThreads, 2) trace_bwd_kernel(const __gri
         const uint2 *st = V.state == nullptr ? nullptr
                           : V.state + (on ? (size_t)c * V.W * V.H + p : 0);
         if (__any_sync(0xffffffffu, on))
-          cone_adjoint<DT, BR, kVar, AN>(L, s_code_off, s_rows[threadIdx.x >> 5], s_lut, on, A, w, cc, T0, g0, g1, g2, ga,
-                                         st, mode);
+          cone_adjoint<DT, BR, kVar, AN>(L, s_code_off, s_rows[threadIdx.x >> 5], s_lut, on, A, w,
+                                         cc, T0, g0, g1, g2, ga, st, mode);
       }
     }
   }

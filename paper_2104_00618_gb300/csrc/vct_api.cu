@@ -707,7 +707,8 @@ static vct_status trace_impl(const vct_pyramid *pyrs, int32_t n_pyr, const vct_v
       if (cfg.ctas_per_sm == 0 && threads == kFwdThreads && cfg.tile_w * cfg.tile_h >= 192 &&
           pyrs[views[v0].pyramid].dtype == VCT_F32 && !bricks && !aniso && !params->flags) {
         threads = kFwdThreads / 2;
-        grid = std::max(1, std::min(2 * grid, (L->total_tiles + threads / 32 - 1) / (threads / 32)));
+        grid = std::max(1, std::min(2 * grid,
+                                    (L->total_tiles + threads / 32 - 1) / (threads / 32)));
       }
     }
     if (v0 > 0 && (e = cudaMemsetAsync(L->queue, 0, 4, stream)) != cudaSuccess)
@@ -876,7 +877,9 @@ vct_status trace_backward_impl(const vct_pyramid *pyr, const vct_view *views,
   // reproducible mode, whose rounds cost more).  Measured on a 64^3 grid
   // with 8 cones, 8 x 8 / 8 x 4 tiles, each cone an item: 5917 pixels 302 /
   // 223 us (reproducible 797 / 448), 32 400: 424 / 355 (718 / 449), 57 600:
-  // 420 / 451 (729 / 513), 129 600: 769 / 823 (875 / 849).
+  // 420 / 451 (729 / 513), 129 600: 769 / 823 (875 / 849).  Either tile gives
+  // a warp's rounds the same 8 x 4 pixels, so the reproducible mode's bits do
+  // not depend on the choice.
   const bool few = pixels < 32 * (deterministic ? resident : resident / 2);
   vct_launch_config c = cfg ? *cfg : vct_launch_config{8, few ? 4 : 8, 1, 0};
   if (!cfg_ok(c)) return fail(VCT_ERR_INVALID_ARG, "vct_trace_backward: bad launch config");

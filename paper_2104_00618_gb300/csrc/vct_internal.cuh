@@ -15,9 +15,11 @@ constexpr int kTraceThreads = 256;      // CTA shape of the adjoint trace kernel
 // Forward trace CTAs: warps work independently, so the CTA size sets the
 // register budget, 65536 / (kFwdThreads * kTraceMinBlocks) per thread, and the
 // copies of the Morton tables per SM: one CTA of 512 threads leaves 24 KB more
-// to the L1 than two of 256 (binary16 128^3 frame 2.51 -> 2.37 ms, anisotropic
-// 3.03 -> 2.87).  Large tiles of dense float32 frames take two all the same
-// (vct_trace's launch has the figures).
+// to the L1 than two of 256 (two scenes each: binary16 128^3, 1111 x 699, 2.77
+// -> 2.69 ms; anisotropic 128^3, 960 x 540, 3.37 -> 3.20; bricks 512^3, 1280 x
+// 720, 4.78 -> 4.72; float32 256^3, 1280 x 720, 3.00 -> 3.01).  Large tiles of
+// dense float32 frames take two all the same (vct_trace's launch has the
+// figures).
 #ifndef VCT_FWD_THREADS
 #define VCT_FWD_THREADS 512
 #endif
